@@ -138,6 +138,7 @@ struct cllm_ctx {
   float2* rope = nullptr;
   float* part_o = nullptr;
   float2* part_ml = nullptr;
+  int* attn_tickets = nullptr;  // fp32 attention: chunks done per (query tile, head)
   float* gemm_part = nullptr;
   size_t gemm_part_elems = 0;
   int* tickets = nullptr;
@@ -344,7 +345,7 @@ cudaError_t gemm(cllm_ctx* c, cudaStream_t s, bool pdl, int kind, int mtiles, in
     EpiArgs ee = e;
     ee.am_units = mtiles * g.ntiles;
     ee.am_mtiles = mtiles;
-    err = launch_gemm_simt(kind, g, ee, s, pdl);
+    err = launch_gemm_f32(kind, g, ee, s, pdl);
   } else {
     EpiArgs ee = e;
     Part p;
@@ -462,13 +463,15 @@ cudaError_t record_forward(cllm_ctx* c, cudaStream_t s, const FwdSpec& f, bool p
     aa.v_cache = vl;
     {
       const int kv_row0 = static_cast<int>(static_cast<size_t>(l) * c->layer_kv_elems / c->hd);
-      const cudaError_t la = c->attn_maps_ok
-                                 ? launch_attention_tma(aa, c->attn_maps, kv_row0, f.attn_grid, s, pdl)
-                                 : launch_attention(aa, ab, f.attn_grid, s, pdl);
+      const cudaError_t la =
+          !c->bf16 ? launch_attention_f32(aa, c->attn_tickets, f.attn_grid, s, pdl)
+          : c->attn_maps_ok ? launch_attention_tma(aa, c->attn_maps, kv_row0, f.attn_grid, s, pdl)
+                            : launch_attention(aa, f.attn_grid, s, pdl);
       if ((err = after_launch(c, s, "attention", la)) != cudaSuccess) return err;
     }
-    if ((err = after_launch(c, s, "attn_combine", launch_attn_combine(aa, ab, s, pdl))) !=
-        cudaSuccess)
+    // (the fp32 kernel merges its own chunks)
+    if (c->bf16 &&
+        (err = after_launch(c, s, "attn_combine", launch_attn_combine(aa, s, pdl))) != cudaSuccess)
       return err;
     // (a4) O-proj + residual; leaves the MLP norm's input and statistics
     e = base_epi(c, T);
@@ -1177,6 +1180,9 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
         rc = CLLM_ECUDA;
         break;
       }
+    } else if (f32_set_attributes() != cudaSuccess) {
+      rc = CLLM_ECUDA;
+      break;
     }
     // capacities
     const int step_rows = a.max_batch * a.max_block;
@@ -1235,7 +1241,8 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
     }
     // attention partials: rows x heads x chunks
     const size_t prow = T * c->H * c->nch_max;
-    ok = dev_alloc(c, &c->part_o, prow * c->hd * 4) && dev_alloc(c, &c->part_ml, prow * 8);
+    ok = dev_alloc(c, &c->part_o, prow * c->hd * 4) && dev_alloc(c, &c->part_ml, prow * 8) &&
+         (c->bf16 || dev_alloc(c, &c->attn_tickets, static_cast<size_t>(c->max_qtiles) * c->H * 4));
     // GEMM split-K partials (T <= 256 launches)
     const int mt_list[5] = {(c->dq + 2 * c->dkv) / kBM, c->d / kBM, ceil_div(c->F, 64), c->d / kBM,
                             ceil_div(c->V, kBM)};

@@ -16,10 +16,8 @@
 // m16n8k16 f16 x f16 -> fp32 with
 // ldmatrix loads from padded shared memory; the softmax is computed on the
 // accumulator fragments with quad shuffles; the 4 warps' partials are merged
-// in warp order.  fp32: a SIMT kernel with a per-row online softmax.
+// in warp order.  (The fp32 engine's attention is in fp32.cu.)
 #include <float.h>
-
-#include <type_traits>
 
 #include "act.cuh"
 #include "attn_item.cuh"
@@ -79,80 +77,15 @@ __global__ void __launch_bounds__(128) attn_chunk_tma_kernel(const __grid_consta
   }
 }
 
-// fp32 (and generic) path: one warp per row, online softmax over the chunk.
-template <typename Act, int HD>
-__global__ void __launch_bounds__(128) attn_chunk_simt_kernel(const AttnArgs a) {
-  __shared__ int pre[kMaxQTilesSmem + 1];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int total = attn_item_prefix(a, pre, threadIdx.x, CtaSync{}, 1);
-  const int group = a.H / a.Hkv;
-  const int ldq = a.H * HD;
-  constexpr int DPL = HD / 32;
-  const Act* Q = static_cast<const Act*>(a.q);
-  const Act* KC = static_cast<const Act*>(a.k_cache);
-  const Act* VC = static_cast<const Act*>(a.v_cache);
-  for (int item = blockIdx.x; item < total; item += gridDim.x) {
-    const int qi = attn_find_qtile(pre, a.n_qtiles, item);
-    const int local = item - pre[qi];
-    const int c = local / a.H, h = local - c * a.H;
-    const int2 qt = a.qtiles[qi];
-    const int b = qt.x, r0 = qt.y;
-    const int nr = min(kQTile, a.seq_nrows[b] - r0);
-    const int start = a.seq_start[b];
-    const int row_g0 = a.seq_row0[b] + r0;
-    const int kb = c * kAttnChunk;
-    const int kvh = h / group;
-    const size_t kvbase = ((static_cast<size_t>(b) * a.Hkv + kvh) * a.max_seq) * HD;
-    for (int i = warp; i < nr; i += 4) {
-      const int pos = start + r0 + i;
-      int kend = min(kb + kAttnChunk, pos + 1);
-      if (kend > a.max_seq) {
-        if (lane == 0) atomicOr(a.err, DERR_CAPACITY);
-        kend = a.max_seq;
-      }
-      float q[DPL], o[DPL];
-#pragma unroll
-      for (int u = 0; u < DPL; ++u) {
-        q[u] = ld_act(Q, static_cast<size_t>(row_g0 + i) * ldq + h * HD + lane + 32 * u);
-        o[u] = 0.f;
-      }
-      float m = -INFINITY, l = 0.f;
-      for (int key = kb; key < kend; ++key) {
-        const size_t off = kvbase + static_cast<size_t>(key) * HD;
-        float dot = 0.f;
-#pragma unroll
-        for (int u = 0; u < DPL; ++u) dot += q[u] * ld_act(KC, off + lane + 32 * u);
-        const float s = warp_sum(dot) * a.scale_log2;
-        const float mn = fmaxf(m, s);
-        const float corr = exp2f(m - mn);  // m = -inf on the first key: corr = 0
-        const float p = exp2f(s - mn);
-        l = l * corr + p;
-#pragma unroll
-        for (int u = 0; u < DPL; ++u) o[u] = o[u] * corr + p * ld_act(VC, off + lane + 32 * u);
-        m = mn;
-      }
-      const size_t pidx = (static_cast<size_t>(row_g0 + i) * a.H + h) * a.nch_max + c;
-#pragma unroll
-      for (int u = 0; u < DPL; ++u) a.part_o[pidx * HD + lane + 32 * u] = o[u];
-      if (lane == 0) a.part_ml[pidx] = (kend > kb) ? make_float2(m, l) : make_float2(-INFINITY, 0.f);
-    }
-  }
-}
-
 // Merge of a row's partials (per chunk range) in order; out = O / l
 // (fmaf accumulation in chunk order, as in the persistent kernel's merge).
 // One (row, head) per hd/4 threads, 4 consecutive dims per thread (vector
 // loads and stores); per element the same sums in the same order as a
 // per-element loop.
-template <typename Act>
 __global__ void __launch_bounds__(128) attn_combine_kernel(const AttnArgs a) {
   pdl_launch_dependents();
   pdl_wait();
-  // the tensor-core path leaves one partial per range of kAttnRange chunks,
-  // the fp32 path one per chunk
-  constexpr int R = std::is_same<Act, float>::value ? 1 : kAttnRange;
+  constexpr int R = kAttnRange;  // one partial per range of kAttnRange chunks
   const int tpp = a.hd / 4;  // threads per (row, head)
   const int pair = blockIdx.x * (blockDim.x / tpp) + threadIdx.x / tpp;
   if (pair >= a.T * a.H) return;
@@ -174,14 +107,13 @@ __global__ void __launch_bounds__(128) attn_combine_kernel(const AttnArgs a) {
     acc.z = fmaf(f, o.z, acc.z);
     acc.w = fmaf(f, o.w, acc.w);
   }
-  st_gin4(static_cast<Act*>(a.out), static_cast<size_t>(t) * a.H * a.hd + h * a.hd + d, a.plane_out,
+  st_gin4(static_cast<__nv_bfloat16*>(a.out), static_cast<size_t>(t) * a.H * a.hd + h * a.hd + d, a.plane_out,
           make_float4(acc.x / l, acc.y / l, acc.z / l, acc.w / l));
 }
 
 // ---- launchers ----------------------------------------------------------------------
 
-size_t attention_smem_bytes(int act_bf16, int hd) {
-  if (!act_bf16) return 0;
+size_t attention_smem_bytes(int hd) {
   return hd == 64 ? sizeof(AttnSmemF16<64>) : sizeof(AttnSmemF16<128>);
 }
 
@@ -220,19 +152,13 @@ static void attn_cfg(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3 gr
   cfg.numAttrs = 1;
 }
 
-cudaError_t launch_attention(const AttnArgs& a, int act_bf16, int grid, cudaStream_t s, bool pdl) {
+cudaError_t launch_attention(const AttnArgs& a, int grid, cudaStream_t s, bool pdl) {
   if (a.n_qtiles > kMaxQTilesSmem) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  if (act_bf16) {
-    attn_cfg(cfg, attr, dim3(grid), dim3(128), attention_smem_bytes(1, a.hd), s, pdl);
-    if (a.hd == 64) return cudaLaunchKernelEx(&cfg, attn_chunk_mma_kernel<64>, a);
-    if (a.hd == 128) return cudaLaunchKernelEx(&cfg, attn_chunk_mma_kernel<128>, a);
-    return cudaErrorInvalidValue;
-  }
-  attn_cfg(cfg, attr, dim3(grid), dim3(128), 0, s, pdl);
-  if (a.hd == 64) return cudaLaunchKernelEx(&cfg, attn_chunk_simt_kernel<float, 64>, a);
-  if (a.hd == 128) return cudaLaunchKernelEx(&cfg, attn_chunk_simt_kernel<float, 128>, a);
+  attn_cfg(cfg, attr, dim3(grid), dim3(128), attention_smem_bytes(a.hd), s, pdl);
+  if (a.hd == 64) return cudaLaunchKernelEx(&cfg, attn_chunk_mma_kernel<64>, a);
+  if (a.hd == 128) return cudaLaunchKernelEx(&cfg, attn_chunk_mma_kernel<128>, a);
   return cudaErrorInvalidValue;
 }
 
@@ -252,13 +178,12 @@ cudaError_t launch_attention_tma(const AttnArgs& a, const AttnMaps& m, int kv_ro
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_attn_combine(const AttnArgs& a, int act_bf16, cudaStream_t s, bool pdl) {
+cudaError_t launch_attn_combine(const AttnArgs& a, cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   const int per_block = 128 / (a.hd / 4);  // (row, head) pairs per 128-thread block
   attn_cfg(cfg, attr, dim3((a.T * a.H + per_block - 1) / per_block), dim3(128), 0, s, pdl);
-  if (act_bf16) return cudaLaunchKernelEx(&cfg, attn_combine_kernel<__nv_bfloat16>, a);
-  return cudaLaunchKernelEx(&cfg, attn_combine_kernel<float>, a);
+  return cudaLaunchKernelEx(&cfg, attn_combine_kernel, a);
 }
 
 }  // namespace cllm

@@ -124,73 +124,6 @@ __global__ void __launch_bounds__(64 + 128 * solo_groups<KIND, BNMAX>(), 1)
 }
 
 // ---------------------------------------------------------------------------------
-// SIMT kernel (fp32 weights and activations; the fp32 parity configuration)
-// One CTA computes a 128-row x 16-token tile over the full K, then runs the
-// same epilogue.
-// ---------------------------------------------------------------------------------
-
-template <int KIND>
-__global__ void __launch_bounds__(128) gemm_simt_kernel(const GemmArgs g, const EpiArgs e) {
-  __shared__ float xs[kEpiCols][kBK + 1];
-  __shared__ EpiSmem es;
-  pdl_launch_dependents();
-  pdl_wait();
-  const int mt = blockIdx.x, nt = blockIdx.y, r = threadIdx.x;
-  const int t0 = nt * kEpiCols;
-  const float* W;
-  int row;
-  bool vrow;
-  if (KIND == EPI_GATEUP) {
-    W = static_cast<const float*>(r < 64 ? g.A0 : g.A1);
-    row = mt * 64 + (r & 63);
-    vrow = row < g.M;
-  } else if (KIND == EPI_QKV) {
-    const int m = mt * kBM + r;
-    if (m < g.rows_q) {
-      W = static_cast<const float*>(g.A0);
-      row = m;
-    } else if (m < g.rows_qk) {
-      W = static_cast<const float*>(g.A1);
-      row = m - g.rows_q;
-    } else {
-      W = static_cast<const float*>(g.A2);
-      row = m - g.rows_qk;
-    }
-    vrow = m < g.M;
-  } else {
-    W = static_cast<const float*>(g.A0);
-    row = mt * kBM + r;
-    vrow = row < g.M;
-  }
-  const float* X = static_cast<const float*>(g.X);
-  float acc[kEpiCols];
-#pragma unroll
-  for (int j = 0; j < kEpiCols; ++j) acc[j] = 0.f;
-  for (int k0 = 0; k0 < g.K; k0 += kBK) {
-    for (int i = r; i < kEpiCols * kBK; i += 128) {
-      const int j = i / kBK, kk = i - j * kBK;
-      const int t = t0 + j, k = k0 + kk;
-      xs[j][kk] = (t < g.T && k < g.K) ? X[static_cast<size_t>(t) * g.ldx + k] : 0.f;
-    }
-    __syncthreads();
-    if (vrow) {
-      const int kend = min(kBK, g.K - k0);
-      const float* wr = W + static_cast<size_t>(row) * g.K + k0;
-      for (int kk = 0; kk < kend; ++kk) {
-        const float w = wr[kk];
-#pragma unroll
-        for (int j = 0; j < kEpiCols; ++j) acc[j] = fmaf(w, xs[j][kk], acc[j]);
-      }
-    }
-    __syncthreads();
-  }
-  if (r == 0) es.prepared = 0;
-  __syncthreads();
-  epi_apply<KIND, float>(e, mt, t0, acc, r, es);
-  if (KIND == EPI_ARGMAX) epi_argmax_finish(e, r, es);
-}
-
-// ---------------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------------
 
@@ -281,25 +214,6 @@ cudaError_t launch_gemm_tc(int kind, int bn_max, const GemmMaps& maps, const Gem
     case EPI_GATEUP: return launch_tc_kind<EPI_GATEUP>(bn_max, maps, g, e, grid, s, pdl);
     case EPI_RESID: return launch_tc_kind<EPI_RESID>(bn_max, maps, g, e, grid, s, pdl);
     case EPI_ARGMAX: return launch_tc_kind<EPI_ARGMAX>(bn_max, maps, g, e, grid, s, pdl);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-template <int KIND>
-static cudaError_t launch_simt_one(const GemmArgs& g, const EpiArgs& e, cudaStream_t s, bool pdl) {
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[1];
-  fill_launch(cfg, attr, dim3(g.mtiles, g.ntiles), dim3(128), 0, s, pdl);
-  return cudaLaunchKernelEx(&cfg, gemm_simt_kernel<KIND>, g, e);
-}
-
-cudaError_t launch_gemm_simt(int kind, const GemmArgs& g, const EpiArgs& e, cudaStream_t s,
-                             bool pdl) {
-  switch (kind) {
-    case EPI_QKV: return launch_simt_one<EPI_QKV>(g, e, s, pdl);
-    case EPI_GATEUP: return launch_simt_one<EPI_GATEUP>(g, e, s, pdl);
-    case EPI_RESID: return launch_simt_one<EPI_RESID>(g, e, s, pdl);
-    case EPI_ARGMAX: return launch_simt_one<EPI_ARGMAX>(g, e, s, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

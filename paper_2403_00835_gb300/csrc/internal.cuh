@@ -91,7 +91,7 @@ struct GemmArgs {
   int pre_stages;       // weight tiles issued before the phase's dependency is met (<= ring)
   float* partial;       // [units*maxc][bn][128] split-K partial tiles
   int* tickets;         // [units] arrival counters (self-resetting)
-  // SIMT (fp32) path only
+  // fp32 path only
   const void* A0;
   const void* A1;
   const void* A2;
@@ -298,14 +298,16 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, 
 cudaError_t launch_embed(const EmbedArgs& a, int act_bf16, cudaStream_t s, bool pdl);
 cudaError_t launch_gemm_tc(int kind, int bn_max, const GemmMaps& maps, const GemmArgs& g,
                            const EpiArgs& e, int grid, cudaStream_t s, bool pdl);
-cudaError_t launch_gemm_simt(int kind, const GemmArgs& g, const EpiArgs& e, cudaStream_t s,
-                             bool pdl);
-cudaError_t launch_attention(const AttnArgs& a, int act_bf16, int grid, cudaStream_t s, bool pdl);
+cudaError_t launch_attention(const AttnArgs& a, int grid, cudaStream_t s, bool pdl);
 // bf16 engine with tensor maps: Q, K and V tiles by TMA (kv_row0: the layer's
 // first cache row in the maps)
 cudaError_t launch_attention_tma(const AttnArgs& a, const AttnMaps& m, int kv_row0, int grid,
                                  cudaStream_t s, bool pdl);
-cudaError_t launch_attn_combine(const AttnArgs& a, int act_bf16, cudaStream_t s, bool pdl);
+cudaError_t launch_attn_combine(const AttnArgs& a, cudaStream_t s, bool pdl);
+// fp32 engine (fp32.cu); tickets: [query tiles][heads], zero, self-resetting
+cudaError_t launch_gemm_f32(int kind, const GemmArgs& g, const EpiArgs& e, cudaStream_t s, bool pdl);
+cudaError_t launch_attention_f32(const AttnArgs& a, int* tickets, int grid, cudaStream_t s, bool pdl);
+cudaError_t f32_set_attributes();
 cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_decode_init(const AcceptArgs& a, cudaStream_t s);
 cudaError_t launch_set_head(int* block, const int* head, int B, int n, int V, int* err,
@@ -318,6 +320,6 @@ int gemm_tc_stages(int bn_max);
 size_t gemm_tc_smem_bytes(int bn_max);
 cudaError_t gemm_tc_set_attributes();
 cudaError_t attention_set_attributes();
-size_t attention_smem_bytes(int act_bf16, int hd);
+size_t attention_smem_bytes(int hd);
 
 }  // namespace cllm
