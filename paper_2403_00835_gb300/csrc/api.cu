@@ -101,6 +101,7 @@ namespace {
 struct LayerW {
   const void *attn_norm, *wq, *wk, *wv, *wo, *mlp_norm, *w_gate, *w_up, *w_down;
   CUtensorMap mq, mk, mv, mo, mgate, mup, mdown;
+  CUtensorMap mq_half, mk_half, mv_half;  // boxes of half a head (wide launches)
 };
 
 enum Mode { MODE_PREFILL = 0, MODE_STEP = 1, MODE_DECODE = 2 };
@@ -142,6 +143,9 @@ struct cllm_ctx {
   float* gemm_part = nullptr;
   size_t gemm_part_elems = 0;
   int* tickets = nullptr;
+  int wide_cl = 0, wide_clusters = 0;  // wide GEMM launches: cluster size, resident clusters
+  float* wide_part = nullptr;          // one split-K partial per CTA
+  int* wide_tickets = nullptr;
   int max_mtiles = 0;
   float* am_part = nullptr;
   int* am_ticket = nullptr;
@@ -348,6 +352,19 @@ cudaError_t gemm(cllm_ctx* c, cudaStream_t s, bool pdl, int kind, int mtiles, in
     err = launch_gemm_f32(kind, g, ee, s, pdl);
   } else {
     EpiArgs ee = e;
+    if (T > 256) {
+      const WidePlan w = plan_wide(kind, M, K, T, c->wide_cl, c->wide_clusters, true);
+      w.apply(g);
+      g.partial = c->wide_part;
+      g.tickets = c->wide_tickets;
+      ee.am_mtiles = mtiles;
+      GemmMaps maps{*m0, m1 ? *m1 : *m0, m2 ? *m2 : *m0, {}};
+      if (!make_map(&maps.b, X, static_cast<uint64_t>(K), static_cast<uint64_t>(2 * c->Tcap),
+                    static_cast<uint32_t>(w.bn)))
+        return cudaErrorInvalidValue;
+      if (kind == EPI_ARGMAX) c->rec_count++;  // its reduction kernel
+      return after_launch(c, s, name, launch_gemm_wide(kind, w.cl, maps, g, ee, w.clusters, s, pdl));
+    }
     Part p;
     g = tc_gemm_args(c, mtiles, M, K, T, ee, &p);
     if (static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM > c->gemm_part_elems && p.ntiles == 1)
@@ -455,8 +472,10 @@ cudaError_t record_forward(cllm_ctx* c, cudaStream_t s, const FwdSpec& f, bool p
     e.k_cache = kl;
     e.v_cache = vl;
     const int Mqkv = c->dq + 2 * c->dkv;
-    if ((err = gemm(c, s, pdl, EPI_QKV, Mqkv / kBM, Mqkv, c->d, T, c->xg, L.wq, L.wk, L.wv, &L.mq,
-                    &L.mk, &L.mv, e, "gemm_qkv")) != cudaSuccess)
+    const bool wide = T > 256;
+    if ((err = gemm(c, s, pdl, EPI_QKV, Mqkv / kBM, Mqkv, c->d, T, c->xg, L.wq, L.wk, L.wv,
+                    wide ? &L.mq_half : &L.mq, wide ? &L.mk_half : &L.mk, wide ? &L.mv_half : &L.mv, e,
+                    "gemm_qkv")) != cudaSuccess)
       return err;
     // (a3) block attention, split over position-anchored key chunks
     aa.k_cache = kl;
@@ -1169,14 +1188,23 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
         ok = make_map(&L.mq, L.wq, c->d, c->dq, kBM) && make_map(&L.mk, L.wk, c->d, c->dkv, kBM) &&
              make_map(&L.mv, L.wv, c->d, c->dkv, kBM) && make_map(&L.mo, L.wo, c->dq, c->d, kBM) &&
              make_map(&L.mgate, L.w_gate, c->d, c->F, 64) && make_map(&L.mup, L.w_up, c->d, c->F, 64) &&
-             make_map(&L.mdown, L.w_down, c->F, c->d, kBM);
+             make_map(&L.mdown, L.w_down, c->F, c->d, kBM) &&
+             make_map(&L.mq_half, L.wq, c->d, c->dq, c->hd / 2) &&
+             make_map(&L.mk_half, L.wk, c->d, c->dkv, c->hd / 2) &&
+             make_map(&L.mv_half, L.wv, c->d, c->dkv, c->hd / 2);
       }
       if (!ok) {
         rc = CLLM_EINVAL;
         break;
       }
       if (gemm_tc_set_attributes() != cudaSuccess || attention_set_attributes() != cudaSuccess ||
-          step_persistent_set_attributes() != cudaSuccess) {
+          step_persistent_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess) {
+        rc = CLLM_ECUDA;
+        break;
+      }
+      c->wide_cl = kWideCluster;
+      c->wide_clusters = gemm_wide_clusters(c->wide_cl);
+      if (c->wide_clusters < 1) {
         rc = CLLM_ECUDA;
         break;
       }
@@ -1256,6 +1284,10 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
       c->max_mtiles = std::max(c->max_mtiles, mt_list[i]);
     }
     c->gemm_part_elems = need;
+    if (c->bf16 && c->Tcap > 256) {
+      const size_t ctas = static_cast<size_t>(c->wide_clusters) * c->wide_cl;
+      ok = ok && dev_alloc(c, &c->wide_part, ctas * kWidePartFloats * 4) && dev_alloc(c, &c->wide_tickets, ctas * 4);
+    }
     ok = ok && dev_alloc(c, &c->gemm_part, need * 4) && dev_alloc(c, &c->tickets, c->max_mtiles * 4) &&
          dev_alloc(c, &c->am_part, static_cast<size_t>(ceil_div(c->V, kBM)) * T * 12) &&
          dev_alloc(c, &c->am_ticket, 16) && dev_alloc(c, &c->pred, T * 4) &&
@@ -1400,7 +1432,7 @@ extern "C" int cllm_prefill(cllm_ctx* c, int B, const int32_t* tokens, const int
         return CLLM_ECUDA;
     }
     c->rec_names = nullptr;
-    if (record_forward(c, c->stream, f, false) != cudaSuccess) return CLLM_ECUDA;
+    if (record_forward(c, c->stream, f, true) != cudaSuccess) return CLLM_ECUDA;
     std::vector<int> pr(f.n_last);
     if (cudaMemcpyAsync(pr.data(), c->pred, f.n_last * 4, cudaMemcpyDeviceToHost, c->stream))
       return CLLM_ECUDA;
@@ -1455,7 +1487,7 @@ extern "C" int cllm_jacobi_step(cllm_ctx* c, const int32_t* guess, int n, int32_
     f.attn_grid = attn_grid_for(c, f.n_qtiles);
     f.want_logits = true;
     f.acc = make_accept(c, B, n, false);
-    if (record_forward(c, c->stream, f, false) != cudaSuccess) return CLLM_ECUDA;
+    if (record_forward(c, c->stream, f, true) != cudaSuccess) return CLLM_ECUDA;
   } else {
     // the persistent kernel of the decode loop; with logits_out its LM-head
     // phase also stores the logits
@@ -1805,12 +1837,20 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
   if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
     return CLLM_ECUDA;
   if (prop.major != 10 || prop.minor != 3) return CLLM_EUNSUPPORTED;
-  if (!get_encode() || gemm_tc_set_attributes() != cudaSuccess) return CLLM_ECUDA;
+  if (!get_encode() || gemm_tc_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess)
+    return CLLM_ECUDA;
   const int mtiles = M / kBM;
   const Part p = plan_gemm(mtiles, K, T, prop.multiProcessorCount);
   const int ldt = round_up(T, 16);
+  const bool wide = T > 256;
+  WidePlan w{};
+  if (wide) {
+    const int clusters = gemm_wide_clusters(kWideCluster);
+    if (clusters < 1) return CLLM_ECUDA;
+    w = plan_wide(EPI_RESID, M, K, T, kWideCluster, clusters, true);
+  }
   GemmMaps maps{};
-  if (!make_map(&maps.a0, W, K, M, kBM) || !make_map(&maps.b, X, K, 2 * x_rows, p.bn))
+  if (!make_map(&maps.a0, W, K, M, kBM) || !make_map(&maps.b, X, K, 2 * x_rows, wide ? w.bn : p.bn))
     return CLLM_EINVAL;
   maps.a1 = maps.a2 = maps.a0;
   std::vector<void*> tmp;
@@ -1822,8 +1862,10 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
   };
   int rc = CLLM_OK;
   do {
-    float* part = static_cast<float*>(alloc(static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
-    int* tickets = static_cast<int*>(alloc(mtiles * 4));
+    const size_t ctas = static_cast<size_t>(w.clusters) * w.cl;
+    float* part = static_cast<float*>(
+        alloc(wide ? ctas * kWidePartFloats * 4 : static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
+    int* tickets = static_cast<int*>(alloc(wide ? ctas * 4 : mtiles * 4));
     int* err = static_cast<int*>(alloc(16));
     float* ssq = static_cast<float*>(alloc(static_cast<size_t>(mtiles) * ldt * 4));
     void* xg = alloc(static_cast<size_t>(T) * M * 2 * 2);
@@ -1852,6 +1894,7 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
     g.lo_rows = x_rows;
     g.l2_ahead = kL2AheadDefault;
     g.pre_stages = 1 << 20;
+    if (wide) w.apply(g);
     g.partial = part;
     g.tickets = tickets;
     g.err = err;
@@ -1865,8 +1908,9 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
     e.ssq_out = ssq;
     e.d = M;
     e.err = err;
-    if (launch_gemm_tc(EPI_RESID, p.bn_max, maps, g, e, p.grid, 0, false) != cudaSuccess ||
-        cudaDeviceSynchronize() != cudaSuccess) {
+    const cudaError_t le = wide ? launch_gemm_wide(EPI_RESID, w.cl, maps, g, e, w.clusters, 0, false)
+                                : launch_gemm_tc(EPI_RESID, p.bn_max, maps, g, e, p.grid, 0, false);
+    if (le != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
       rc = CLLM_ECUDA;
       break;
     }

@@ -295,6 +295,32 @@ Part plan_gemm(int mtiles, int K, int T, int sms);
 // bf16 [outer][inner] tensor map: 64-column x box_outer-row tiles, 128-byte swizzle.
 bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint32_t box_outer);
 
+
+// Wide launches (T > 256, gemm_wide.cu): units of 512 weight rows (gate/up:
+// 256 features) x bn tokens per CTA pair, the (unit, K chunk) space in ranges
+// of cpc chunks per cluster of cl CTAs.
+constexpr int kWideTokens = 128;                     // most tokens of a pair's tile
+constexpr int kWidePartFloats = 2 * kWideTokens * kBM;  // a CTA's split-K partial
+constexpr int kWideCluster = 4;                      // CTAs per cluster
+struct WidePlan {
+  int cl, row_units, ntiles, bn, kchunks, cpc, clusters;
+  void apply(GemmArgs& g) const {
+    g.mtiles = row_units;
+    g.ntiles = ntiles;
+    g.bn = bn;
+    g.kchunks = kchunks;
+    g.cpc = cpc;
+  }
+};
+// split: ranges may cut a unit (needs kWidePartFloats floats and one zeroed
+// ticket per CTA); otherwise whole units
+WidePlan plan_wide(int kind, int M, int K, int T, int cl, int clusters, bool split);
+int gemm_wide_clusters(int cl);
+cudaError_t gemm_wide_set_attributes();
+// (ARGMAX: two kernels, the second reduces the tiles' maxima)
+cudaError_t launch_gemm_wide(int kind, int cl, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
+                             cudaStream_t s, bool pdl);
+
 cudaError_t launch_embed(const EmbedArgs& a, int act_bf16, cudaStream_t s, bool pdl);
 cudaError_t launch_gemm_tc(int kind, int bn_max, const GemmMaps& maps, const GemmArgs& g,
                            const EpiArgs& e, int grid, cudaStream_t s, bool pdl);

@@ -83,9 +83,19 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   if (rc != CLLM_OK) return rc;
   char* sb = static_cast<char*>(base);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  if (gemm_tc_set_attributes() != cudaSuccess) return CLLM_ECUDA;
+  // T > 256: whole units, which need no partials
+  const bool wide = T > 256;
+  WidePlan w{};
+  if (wide) {
+    if (gemm_wide_set_attributes() != cudaSuccess) return CLLM_ECUDA;
+    const int clusters = gemm_wide_clusters(kWideCluster);
+    if (clusters < 1) return CLLM_ECUDA;
+    w = plan_wide(EPI_RESID, M, K, T, kWideCluster, clusters, false);
+  } else if (gemm_tc_set_attributes() != cudaSuccess) {
+    return CLLM_ECUDA;
+  }
   GemmMaps maps{};
-  if (!make_map(&maps.a0, W, K, M, kBM) || !make_map(&maps.b, X, K, 2 * x_rows, p.bn))
+  if (!make_map(&maps.a0, W, K, M, kBM) || !make_map(&maps.b, X, K, 2 * x_rows, wide ? w.bn : p.bn))
     return CLLM_EINVAL;
   maps.a1 = maps.a2 = maps.a0;
   // the array keeps the previous call's contents: tickets and the error word
@@ -111,6 +121,7 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   g.lo_rows = x_rows;
   g.l2_ahead = kL2AheadDefault;  // as the allocating GEMM entry points
   g.pre_stages = 1 << 20;
+  if (wide) w.apply(g);
   g.partial = reinterpret_cast<float*>(sb + off_part);
   g.tickets = reinterpret_cast<int*>(sb + off_tick);
   g.err = reinterpret_cast<int*>(sb + off_err);
@@ -124,8 +135,9 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   e.ssq_out = reinterpret_cast<float*>(sb + off_ssq);
   e.d = M;
   e.err = g.err;
-  if (launch_gemm_tc(EPI_RESID, p.bn_max, maps, g, e, p.grid, s, false) != cudaSuccess)
-    return CLLM_ECUDA;
+  const cudaError_t le = wide ? launch_gemm_wide(EPI_RESID, w.cl, maps, g, e, w.clusters, s, false)
+                              : launch_gemm_tc(EPI_RESID, p.bn_max, maps, g, e, p.grid, s, false);
+  if (le != cudaSuccess) return CLLM_ECUDA;
   int herr = 0;
   if (cudaMemcpyAsync(&herr, g.err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
