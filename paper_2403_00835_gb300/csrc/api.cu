@@ -388,6 +388,8 @@ struct FwdSpec {
   int n_qtiles;
   const int2* qtiles;
   int attn_grid;
+  int n_wtiles;        // > 0: wide attention over these 256-row tiles
+  const int2* wtiles;
   int n_last;  // prefill: rows whose logits are needed (gathered)
   bool want_logits;
   AcceptArgs acc;  // step/decode
@@ -459,6 +461,9 @@ cudaError_t record_forward(cllm_ctx* c, cudaStream_t s, const FwdSpec& f, bool p
   const EmbedArgs ea = make_embed_args(c, f);
   if ((err = after_launch(c, s, "embed", launch_embed(ea, ab, s, pdl))) != cudaSuccess) return err;
   AttnArgs aa = make_attn_args(c, f);
+  AttnArgs aw = aa;  // wide attention
+  aw.qtiles = f.wtiles;
+  aw.n_qtiles = f.n_wtiles;
 
   for (int l = 0; l < c->NL; ++l) {
     const LayerW& L = c->layers[l];
@@ -478,18 +483,19 @@ cudaError_t record_forward(cllm_ctx* c, cudaStream_t s, const FwdSpec& f, bool p
                     "gemm_qkv")) != cudaSuccess)
       return err;
     // (a3) block attention, split over position-anchored key chunks
-    aa.k_cache = kl;
-    aa.v_cache = vl;
+    aa.k_cache = aw.k_cache = kl;
+    aa.v_cache = aw.v_cache = vl;
     {
       const int kv_row0 = static_cast<int>(static_cast<size_t>(l) * c->layer_kv_elems / c->hd);
       const cudaError_t la =
           !c->bf16 ? launch_attention_f32(aa, c->attn_tickets, f.attn_grid, s, pdl)
+          : f.n_wtiles > 0 && f.n_qtiles <= 2048 ? launch_attention_wide(aw, c->attn_maps, kv_row0, s, pdl)
           : c->attn_maps_ok ? launch_attention_tma(aa, c->attn_maps, kv_row0, f.attn_grid, s, pdl)
                             : launch_attention(aa, f.attn_grid, s, pdl);
       if ((err = after_launch(c, s, "attention", la)) != cudaSuccess) return err;
     }
-    // (the fp32 kernel merges its own chunks)
-    if (c->bf16 &&
+    // (the fp32 kernel merges its own chunks; the wide one has no parts to merge)
+    if (c->bf16 && f.n_wtiles == 0 &&
         (err = after_launch(c, s, "attn_combine", launch_attn_combine(aa, s, pdl))) != cudaSuccess)
       return err;
     // (a4) O-proj + residual; leaves the MLP norm's input and statistics
@@ -615,6 +621,26 @@ std::vector<int2> step_qtiles(int B, int n) {
   std::vector<int2> v;
   for (int b = 0; b < B; ++b)
     for (int r0 = 0; r0 < n; r0 += kQTile) v.push_back(make_int2(b, r0));
+  return v;
+}
+
+// 256-row tiles (b, first row) of sequences of nrows[b] rows from position
+// start[b] on, most keys first; empty when the launch's attention runs on
+// 16-row tiles: up to 256 rows (a row's bits must not depend on the launch's
+// width there), or fewer than 64 rows per tile on average (at 64 rows, 16
+// sequences and 320 keys the two take 59 and 48 + 15 us; below that most of a
+// 128-row MMA tile is padding).
+std::vector<int2> wide_tiles(const cllm_ctx* c, const std::vector<int>& start, const std::vector<int>& nrows) {
+  std::vector<int2> v;
+  long T = 0;
+  for (size_t b = 0; b < nrows.size(); ++b) {
+    T += nrows[b];
+    for (int r0 = 0; r0 < nrows[b]; r0 += kWideQTile) v.push_back(make_int2(static_cast<int>(b), r0));
+  }
+  if (!c->attn_maps_ok || T <= 256 || T < 64L * static_cast<long>(v.size())) return {};
+  std::stable_sort(v.begin(), v.end(), [&](const int2& p, const int2& q) {
+    return start[p.x] + std::min(p.y + kWideQTile, nrows[p.x]) > start[q.x] + std::min(q.y + kWideQTile, nrows[q.x]);
+  });
   return v;
 }
 
@@ -858,6 +884,9 @@ int get_graph(cllm_ctx* c, int mode, int n, cllm_ctx::GraphEntry** out) {
   }
   cllm_ctx::GraphEntry ge;
   std::vector<int2> qt = step_qtiles(B, n);
+  const int n_qt = static_cast<int>(qt.size());
+  const std::vector<int2> wt = wide_tiles(c, std::vector<int>(B, 0), std::vector<int>(B, n));
+  qt.insert(qt.end(), wt.begin(), wt.end());
   if (lib_malloc(reinterpret_cast<void**>(&ge.qtiles), qt.size() * sizeof(int2)) != cudaSuccess)
     return CLLM_ENOMEM;
   if (cudaMemcpy(ge.qtiles, qt.data(), qt.size() * sizeof(int2), cudaMemcpyHostToDevice) !=
@@ -870,7 +899,7 @@ int get_graph(cllm_ctx* c, int mode, int n, cllm_ctx::GraphEntry** out) {
     if (!prm) return CLLM_ENOMEM;
     StepArgs& sa = prm->a;
     int bn_max = 32;
-    int rc = build_persistent(c, mode, B, n, ge.qtiles, static_cast<int>(qt.size()), ge, *prm, bn_max);
+    int rc = build_persistent(c, mode, B, n, ge.qtiles, n_qt, ge, *prm, bn_max);
     if (rc != CLLM_OK) {
       cudaFree(ge.qtiles);
       for (void* p : ge.bufs) cudaFree(p);
@@ -968,7 +997,9 @@ int get_graph(cllm_ctx* c, int mode, int n, cllm_ctx::GraphEntry** out) {
   f.B = B;
   f.n = n;
   f.qtiles = ge.qtiles;
-  f.n_qtiles = static_cast<int>(qt.size());
+  f.n_qtiles = n_qt;
+  f.wtiles = ge.qtiles + n_qt;
+  f.n_wtiles = static_cast<int>(wt.size());
   f.attn_grid = attn_grid_for(c, f.n_qtiles);
   f.acc = make_accept(c, B, n, mode == MODE_DECODE);
   cudaGraph_t g = nullptr;
@@ -1198,7 +1229,8 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
         break;
       }
       if (gemm_tc_set_attributes() != cudaSuccess || attention_set_attributes() != cudaSuccess ||
-          step_persistent_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess) {
+          step_persistent_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess ||
+          attention_wide_set_attributes() != cudaSuccess) {
         rc = CLLM_ECUDA;
         break;
       }
@@ -1247,7 +1279,8 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
       c->attn_maps_ok = kv_rows + kAttnChunk < (1ull << 31) &&
                         make_map(&c->attn_maps.k, c->kc, c->hd, kv_rows, kAttnChunk) &&
                         make_map(&c->attn_maps.v, c->vc, c->hd, kv_rows, kAttnChunk) &&
-                        make_map(&c->attn_maps.q, c->q, c->dq, static_cast<uint64_t>(c->Tcap), kQTile);
+                        make_map(&c->attn_maps.q, c->q, c->dq, static_cast<uint64_t>(c->Tcap), kQTile) &&
+                        make_map(&c->attn_maps.qw, c->q, c->dq, static_cast<uint64_t>(c->Tcap), 128);
     }
     // RoPE table (cos, sin) of pos * theta^(-2i/hd), evaluated in double
     {
@@ -1296,7 +1329,8 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
          dev_alloc(c, &c->bidx_in, T * 4) && dev_alloc(c, &c->pos, T * 4) &&
          dev_alloc(c, &c->bidx, T * 4) && dev_alloc(c, &c->seq_start, a.max_batch * 4) &&
          dev_alloc(c, &c->seq_row0, a.max_batch * 4) && dev_alloc(c, &c->seq_nrows, a.max_batch * 4) &&
-         dev_alloc(c, &c->qtiles_prefill, c->max_qtiles * sizeof(int2));
+         dev_alloc(c, &c->qtiles_prefill,
+                   (c->max_qtiles + T / kWideQTile + a.max_batch) * sizeof(int2));
     const size_t Bm = a.max_batch;
     ok = ok && dev_alloc(c, &c->Ld, Bm * 4) && dev_alloc(c, &c->head, Bm * 4) &&
          dev_alloc(c, &c->head0, Bm * 4) && dev_alloc(c, &c->block, Bm * a.max_block * 4) &&
@@ -1397,6 +1431,9 @@ extern "C" int cllm_prefill(cllm_ctx* c, int B, const int32_t* tokens, const int
       }
     }
     const int T = used;
+    const int n_qt = static_cast<int>(qt.size());
+    const std::vector<int2> wt = wide_tiles(c, start, nrows);
+    qt.insert(qt.end(), wt.begin(), wt.end());
     if (cudaMemcpyAsync(c->tok_in, tok.data(), T * 4, cudaMemcpyHostToDevice, c->stream) ||
         cudaMemcpyAsync(c->pos_in, pos.data(), T * 4, cudaMemcpyHostToDevice, c->stream) ||
         cudaMemcpyAsync(c->bidx_in, bidx.data(), T * 4, cudaMemcpyHostToDevice, c->stream) ||
@@ -1415,9 +1452,12 @@ extern "C" int cllm_prefill(cllm_ctx* c, int B, const int32_t* tokens, const int
     f.T = T;
     f.B = B;
     f.qtiles = c->qtiles_prefill;
-    f.n_qtiles = static_cast<int>(qt.size());
+    f.n_qtiles = n_qt;
+    f.wtiles = c->qtiles_prefill + n_qt;
+    f.n_wtiles = static_cast<int>(wt.size());
     long items = 0;
-    for (auto& q : qt) {
+    for (int i = 0; i < n_qt; ++i) {
+      const int2 q = qt[i];
       const int nr = std::min(kQTile, nrows[q.x] - q.y);
       items += static_cast<long>(c->H) * ((start[q.x] + q.y + nr - 1) / kAttnChunk + 1);
     }
@@ -1474,6 +1514,9 @@ extern "C" int cllm_jacobi_step(cllm_ctx* c, const int32_t* guess, int n, int32_
     return CLLM_ECUDA;
   if (logits_out && !persistent_ok(c, B, n)) {
     std::vector<int2> qt = step_qtiles(B, n);
+    const int n_qt = static_cast<int>(qt.size());
+    const std::vector<int2> wt = wide_tiles(c, std::vector<int>(B, 0), std::vector<int>(B, n));
+    qt.insert(qt.end(), wt.begin(), wt.end());
     if (cudaMemcpyAsync(c->qtiles_prefill, qt.data(), qt.size() * sizeof(int2),
                         cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
       return CLLM_ECUDA;
@@ -1483,7 +1526,9 @@ extern "C" int cllm_jacobi_step(cllm_ctx* c, const int32_t* guess, int n, int32_
     f.B = B;
     f.n = n;
     f.qtiles = c->qtiles_prefill;
-    f.n_qtiles = static_cast<int>(qt.size());
+    f.n_qtiles = n_qt;
+    f.wtiles = c->qtiles_prefill + n_qt;
+    f.n_wtiles = static_cast<int>(wt.size());
     f.attn_grid = attn_grid_for(c, f.n_qtiles);
     f.want_logits = true;
     f.acc = make_accept(c, B, n, false);

@@ -281,7 +281,7 @@ struct GemmMaps {
 // of hd values (128-row boxes) and Q (16-row boxes), 64-column halves with the
 // 128-byte swizzle.
 struct AttnMaps {
-  CUtensorMap k, v, q;
+  CUtensorMap k, v, q, qw;  // qw: Q in 128-row boxes (wide attention)
 };
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
@@ -329,6 +329,10 @@ cudaError_t launch_attention(const AttnArgs& a, int grid, cudaStream_t s, bool p
 // first cache row in the maps)
 cudaError_t launch_attention_tma(const AttnArgs& a, const AttnMaps& m, int kv_row0, int grid,
                                  cudaStream_t s, bool pdl);
+// many rows per sequence (attention_wide.cu): a.qtiles = (b, first row) per 256-row tile
+cudaError_t launch_attention_wide(const AttnArgs& a, const AttnMaps& m, int kv_row0, cudaStream_t s, bool pdl);
+cudaError_t attention_wide_set_attributes();
+constexpr int kWideQTile = 256;
 cudaError_t launch_attn_combine(const AttnArgs& a, cudaStream_t s, bool pdl);
 // fp32 engine (fp32.cu); tickets: [query tiles][heads], zero, self-resetting
 cudaError_t launch_gemm_f32(int kind, const GemmArgs& g, const EpiArgs& e, cudaStream_t s, bool pdl);

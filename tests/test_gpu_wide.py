@@ -103,3 +103,34 @@ def test_wide_step_matches_oracle_ragged_vocab():
                 assert r["next"][b][k] == st.pred[k]
             assert abs(r["gap"][b][k] - st.gap[k]) < FLAG_GAP
         s.close()
+
+
+@pytest.mark.parametrize("hd,kv,lens", [
+    (128, 2, [129, 128, 127, 1]), (128, 1, [385]), (64, 4, [256, 257]), (64, 2, [640, 130])])
+def test_wide_attention_matches_oracle_at_tile_edges(hd, kv, lens):
+    """Prompts around the 128-row tiles and 128-key chunks of the wide
+    attention (last tile absent, one row, full), the wide tiles' outputs read
+    back through a short step.  Weights of std 0.08 spread the scores over
+    tens of units, so that running maxima move and accumulators are rescaled."""
+    cfg = replace(syn.TINY_BF16, n_heads=256 // hd, n_kv_heads=kv, head_dim=hd)
+    w_cpu = syn.make_weights(cfg, seed=11, device="cpu")
+    for l in range(cfg.n_layers):
+        for k in ("wq", "wk"):
+            w_cpu[k][l] = w_cpu[k][l] * 4
+    om = oracle_for(cfg, w_cpu)
+    prompts = syn.make_prompts(cfg.vocab, lens, seed=12)
+    n = 3
+    guesses = syn.make_guesses(cfg.vocab, len(lens), n, seed=13)
+    eng = engine_for(cfg, syn.weights_to(w_cpu, "cuda"), max_batch=len(lens), max_seq=max(lens) + 2 * n, max_block=n)
+    try:
+        heads = eng.prefill(prompts)
+        r = eng.jacobi_step(guesses, want_logits=True)
+    finally:
+        eng.close()
+    for b, p in enumerate(prompts):
+        s = om.session(len(p) + n + 1)
+        orc.prefill(s, p)
+        st = orc.jacobi_step(s, [int(heads[b])] + list(guesses[b][1:]), len(p), keep_logits=True)
+        ok, worst = logits_ok(r["logits"][b], st.logits, "bf16")
+        assert ok, (b, worst)
+        s.close()
