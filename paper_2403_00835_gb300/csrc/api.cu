@@ -143,7 +143,7 @@ struct cllm_ctx {
   float* gemm_part = nullptr;
   size_t gemm_part_elems = 0;
   int* tickets = nullptr;
-  int wide_cl = 0, wide_clusters = 0;  // wide GEMM launches: cluster size, resident clusters
+  int wide_clusters = 0;       // wide GEMM launches: resident clusters
   float* wide_part = nullptr;          // one split-K partial per CTA
   int* wide_tickets = nullptr;
   int max_mtiles = 0;
@@ -353,7 +353,7 @@ cudaError_t gemm(cllm_ctx* c, cudaStream_t s, bool pdl, int kind, int mtiles, in
   } else {
     EpiArgs ee = e;
     if (T > 256) {
-      const WidePlan w = plan_wide(kind, M, K, T, c->wide_cl, c->wide_clusters, true);
+      const WidePlan w = plan_wide(kind, M, K, T, c->wide_clusters, true);
       w.apply(g);
       g.partial = c->wide_part;
       g.tickets = c->wide_tickets;
@@ -363,7 +363,7 @@ cudaError_t gemm(cllm_ctx* c, cudaStream_t s, bool pdl, int kind, int mtiles, in
                     static_cast<uint32_t>(w.bn)))
         return cudaErrorInvalidValue;
       if (kind == EPI_ARGMAX) c->rec_count++;  // its reduction kernel
-      return after_launch(c, s, name, launch_gemm_wide(kind, w.cl, maps, g, ee, w.clusters, s, pdl));
+      return after_launch(c, s, name, launch_gemm_wide(kind, maps, g, ee, w.clusters, s, pdl));
     }
     Part p;
     g = tc_gemm_args(c, mtiles, M, K, T, ee, &p);
@@ -1230,12 +1230,12 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
       }
       if (gemm_tc_set_attributes() != cudaSuccess || attention_set_attributes() != cudaSuccess ||
           step_persistent_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess ||
+          gemm_wide_set_attributes_acc() != cudaSuccess ||
           attention_wide_set_attributes() != cudaSuccess) {
         rc = CLLM_ECUDA;
         break;
       }
-      c->wide_cl = kWideCluster;
-      c->wide_clusters = gemm_wide_clusters(c->wide_cl);
+      c->wide_clusters = gemm_wide_clusters();
       if (c->wide_clusters < 1) {
         rc = CLLM_ECUDA;
         break;
@@ -1318,7 +1318,7 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
     }
     c->gemm_part_elems = need;
     if (c->bf16 && c->Tcap > 256) {
-      const size_t ctas = static_cast<size_t>(c->wide_clusters) * c->wide_cl;
+      const size_t ctas = static_cast<size_t>(c->wide_clusters) * kWideCluster;
       ok = ok && dev_alloc(c, &c->wide_part, ctas * kWidePartFloats * 4) && dev_alloc(c, &c->wide_tickets, ctas * 4);
     }
     ok = ok && dev_alloc(c, &c->gemm_part, need * 4) && dev_alloc(c, &c->tickets, c->max_mtiles * 4) &&
@@ -1882,7 +1882,8 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
   if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
     return CLLM_ECUDA;
   if (prop.major != 10 || prop.minor != 3) return CLLM_EUNSUPPORTED;
-  if (!get_encode() || gemm_tc_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess)
+  if (!get_encode() || gemm_tc_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess ||
+      gemm_wide_set_attributes_acc() != cudaSuccess)
     return CLLM_ECUDA;
   const int mtiles = M / kBM;
   const Part p = plan_gemm(mtiles, K, T, prop.multiProcessorCount);
@@ -1890,9 +1891,9 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
   const bool wide = T > 256;
   WidePlan w{};
   if (wide) {
-    const int clusters = gemm_wide_clusters(kWideCluster);
+    const int clusters = gemm_wide_clusters();
     if (clusters < 1) return CLLM_ECUDA;
-    w = plan_wide(EPI_RESID, M, K, T, kWideCluster, clusters, true);
+    w = plan_wide(EPI_RESID, M, K, T, clusters, true);
   }
   GemmMaps maps{};
   if (!make_map(&maps.a0, W, K, M, kBM) || !make_map(&maps.b, X, K, 2 * x_rows, wide ? w.bn : p.bn))
@@ -1907,7 +1908,7 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
   };
   int rc = CLLM_OK;
   do {
-    const size_t ctas = static_cast<size_t>(w.clusters) * w.cl;
+    const size_t ctas = static_cast<size_t>(w.clusters) * kWideCluster;
     float* part = static_cast<float*>(
         alloc(wide ? ctas * kWidePartFloats * 4 : static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
     int* tickets = static_cast<int*>(alloc(wide ? ctas * 4 : mtiles * 4));
@@ -1953,7 +1954,7 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
     e.ssq_out = ssq;
     e.d = M;
     e.err = err;
-    const cudaError_t le = wide ? launch_gemm_wide(EPI_RESID, w.cl, maps, g, e, w.clusters, 0, false)
+    const cudaError_t le = wide ? launch_gemm_wide(EPI_RESID, maps, g, e, w.clusters, 0, false)
                                 : launch_gemm_tc(EPI_RESID, p.bn_max, maps, g, e, p.grid, 0, false);
     if (le != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
       rc = CLLM_ECUDA;

@@ -4,6 +4,7 @@
 //   EPI_GATEUP : x rms-scale, silu(gate) * up -> h
 //   EPI_RESID  : residual add into the fp32 stream, next norm's input and
 //                per-tile sum of squares
+//   EPI_ACC    : the residual add alone
 //   EPI_ARGMAX : x rms-scale, per-tile (max, argmax, 2nd max) of the logits;
 //                the last tile to finish reduces them to argmax and top-2 gap
 #pragma once
@@ -83,7 +84,7 @@ __device__ void epi_prepare(const EpiArgs& e, int r, EpiSmem& s) {
     epi_sync();
     return;
   }
-  if (KIND != EPI_RESID) {
+  if (KIND != EPI_RESID && KIND != EPI_ACC) {
     const int col = r >> 3, part = r & 7;
     for (int t0 = 0; t0 < e.T; t0 += kEpiCols) {
       const int t = t0 + col;
@@ -173,9 +174,9 @@ __device__ __forceinline__ void epi_prefetch(const EpiArgs& e, int mt, int t0, i
                                              const EpiSmem& s, EpiPre& p) {
   p.ok = 0;
   p.t0 = t0;
-  if (KIND == EPI_RESID) {
+  if (KIND == EPI_RESID || KIND == EPI_ACC) {
     const int m = mt * kBM + r;
-    p.g = ld_act(reinterpret_cast<const Act*>(e.gnext), m);
+    if (KIND == EPI_RESID) p.g = ld_act(reinterpret_cast<const Act*>(e.gnext), m);
 #pragma unroll
     for (int j = 0; j < kEpiCols; ++j) {
       const int t = t0 + j;
@@ -311,6 +312,15 @@ __device__ void epi_apply(const EpiArgs& e, int mt, int t0, float (&v)[kEpiCols]
       }
     }
     epi_sync();
+  } else if (KIND == EPI_ACC) {
+    float* xp = e.x + static_cast<size_t>(t0) * e.d + mt * kBM + r;
+    float xi[kEpiCols];
+#pragma unroll
+    for (int j = 0; j < kEpiCols; ++j)
+      xi[j] = use_pre ? pre->a[j] : ((full || t0 + j < e.T) ? __ldcg(xp + static_cast<size_t>(j) * e.d) : 0.f);
+#pragma unroll
+    for (int j = 0; j < kEpiCols; ++j)
+      if (full || t0 + j < e.T) xp[static_cast<size_t>(j) * e.d] = xi[j] + v[j];
   } else if (KIND == EPI_RESID) {
     const int m = mt * kBM + r;
     const float gn = use_pre ? pre->g : ld_act(reinterpret_cast<const Act*>(e.gnext), m);

@@ -173,6 +173,15 @@ cudaError_t gemm_tc_set_attributes() {
   return set_attr_kind<EPI_ARGMAX>();
 }
 
+cudaError_t gemm_tc_set_attributes_acc(int bn_max) {
+  switch (bn_max) {
+    case 32: return set_attr_one<EPI_ACC, 32>();
+    case 64: return set_attr_one<EPI_ACC, 64>();
+    case 128: return set_attr_one<EPI_ACC, 128>();
+    default: return set_attr_one<EPI_ACC, 256>();
+  }
+}
+
 static void fill_launch(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3 grid, dim3 block,
                         size_t smem, cudaStream_t s, bool pdl) {
   cfg = cudaLaunchConfig_t{};
@@ -214,6 +223,7 @@ cudaError_t launch_gemm_tc(int kind, int bn_max, const GemmMaps& maps, const Gem
     case EPI_GATEUP: return launch_tc_kind<EPI_GATEUP>(bn_max, maps, g, e, grid, s, pdl);
     case EPI_RESID: return launch_tc_kind<EPI_RESID>(bn_max, maps, g, e, grid, s, pdl);
     case EPI_ARGMAX: return launch_tc_kind<EPI_ARGMAX>(bn_max, maps, g, e, grid, s, pdl);
+    case EPI_ACC: return launch_tc_kind<EPI_ACC>(bn_max, maps, g, e, grid, s, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -189,14 +189,14 @@ __device__ __forceinline__ void wide_apply(const EpiArgs& e, const GemmArgs& g, 
       }
     }
     if (bad) atomicOr(e.err, DERR_CAPACITY);
-  } else if (KIND == EPI_RESID) {
+  } else if (KIND == EPI_RESID || KIND == EPI_ACC) {
 #pragma unroll
     for (int st = 0; st < 8; ++st) {
       const int a = st >> 2, c = st & 3;
       const int m = row0 + a * kBM + lr, tl = (grp + 2 * c) * kEpiCols;
       if (m >= g.M || tl >= g.bn) continue;  // whole tiles (M is a multiple of 128)
       float (&v)[4][kEpiCols] = a == 0 ? v0 : v1;
-      const float gn = ld_act(static_cast<const __nv_bfloat16*>(e.gnext), m);
+      const float gn = KIND == EPI_RESID ? ld_act(static_cast<const __nv_bfloat16*>(e.gnext), m) : 0.f;
       float* xp = e.x + static_cast<size_t>(t0 + tl) * e.d + m;
       __nv_bfloat16* gp = static_cast<__nv_bfloat16*>(e.xg) + static_cast<size_t>(t0 + tl) * e.d + m;
       float xi[kEpiCols], sq[kEpiCols];
@@ -213,12 +213,14 @@ __device__ __forceinline__ void wide_apply(const EpiArgs& e, const GemmArgs& g, 
         if (live) {
           const size_t o = static_cast<size_t>(j) * e.d;
           xp[o] = xi[j];
-          st_gin(gp, o, e.plane_x, xi[j] * gn);
+          if (KIND == EPI_RESID) st_gin(gp, o, e.plane_x, xi[j] * gn);
         }
       }
+      if (KIND == EPI_ACC) continue;
       const float col = warp_colsum16(sq, lane);
       if ((lane & 1) == 0) s.red[grp][a][c][w4][lane >> 1] = col;
     }
+    if (KIND == EPI_ACC) return;
     named_bar_sync(1 + grp, 128);
     {
       // thread -> (accumulator, chunk, column) of its group's tokens
@@ -492,7 +494,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
     while (work.next(sg, cluster, first, last)) {
       const int t0 = unit_tok(sg.unit), row0 = unit_row(sg.unit);
       const bool owner = cluster == first;
-      if (owner && KIND != EPI_RESID) {
+      if (owner && KIND != EPI_RESID && KIND != EPI_ACC) {
         // the unit's RMSNorm scales, positions and sequences, while its MMAs run
         for (int tb = 0; tb < g.bn; tb += 32) {
           const int tl = tb + (et >> 3), t = t0 + tl;
@@ -610,41 +612,36 @@ static cudaError_t wide_set_one() {
                               static_cast<int>(wide_smem_bytes()));
 }
 
+cudaError_t gemm_wide_set_attributes_acc() { return wide_set_one<EPI_ACC, kWideCluster>(); }
+
 cudaError_t gemm_wide_set_attributes() {
   cudaError_t err;
-  if ((err = wide_set_one<EPI_QKV, 2>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_GATEUP, 2>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_RESID, 2>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_ARGMAX, 2>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_QKV, 4>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_GATEUP, 4>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_RESID, 4>()) != cudaSuccess) return err;
-  return wide_set_one<EPI_ARGMAX, 4>();
+  if ((err = wide_set_one<EPI_QKV, kWideCluster>()) != cudaSuccess) return err;
+  if ((err = wide_set_one<EPI_GATEUP, kWideCluster>()) != cudaSuccess) return err;
+  if ((err = wide_set_one<EPI_RESID, kWideCluster>()) != cudaSuccess) return err;
+  return wide_set_one<EPI_ARGMAX, kWideCluster>();
 }
 
-// Clusters of `cl` CTAs that can be resident at once (0: none, or an error).
-int gemm_wide_clusters(int cl) {
+// Clusters that can be resident at once (0: none, or an error).
+int gemm_wide_clusters() {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
-  cfg.gridDim = dim3(cl * 64);
+  cfg.gridDim = dim3(kWideCluster * 64);
   cfg.blockDim = dim3(kWThreads);
   cfg.dynamicSmemBytes = wide_smem_bytes();
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.x = kWideCluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  const cudaError_t e = cl == 4 ? cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI_RESID, 4>, &cfg)
-                                : cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI_RESID, 2>, &cfg);
-  return e == cudaSuccess ? n : 0;
+  return cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI_ACC, kWideCluster>, &cfg) == cudaSuccess ? n : 0;
 }
 
-WidePlan plan_wide(int kind, int M, int K, int T, int cl, int clusters, bool split) {
+WidePlan plan_wide(int kind, int M, int K, int T, int clusters, bool split) {
   WidePlan p{};
-  const int pairs = cl / 2;
-  p.cl = cl;
+  constexpr int pairs = kWideCluster / 2;
   p.row_units = ceil_div(M, kind == EPI_GATEUP ? 256 : 512);
   p.ntiles = ceil_div(T, kWideTokens * pairs);
   p.bn = round_up(ceil_div(T, p.ntiles * pairs), kEpiCols);
@@ -676,24 +673,18 @@ static cudaError_t launch_wide_one(const GemmMaps& m, const GemmArgs& g, const E
   return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<KIND, CL>, m.a0, m.a1, m.a2, m.b, g, e);
 }
 
-template <int KIND>
-static cudaError_t launch_wide_kind(int cl, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
-                                    cudaStream_t s, bool pdl) {
-  return cl == 4 ? launch_wide_one<KIND, 4>(m, g, e, clusters, s, pdl)
-                 : launch_wide_one<KIND, 2>(m, g, e, clusters, s, pdl);
-}
-
-cudaError_t launch_gemm_wide(int kind, int cl, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
+cudaError_t launch_gemm_wide(int kind, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
                              cudaStream_t s, bool pdl) {
   cudaError_t err;
   switch (kind) {
-    case EPI_QKV: return launch_wide_kind<EPI_QKV>(cl, m, g, e, clusters, s, pdl);
-    case EPI_GATEUP: return launch_wide_kind<EPI_GATEUP>(cl, m, g, e, clusters, s, pdl);
-    case EPI_RESID: return launch_wide_kind<EPI_RESID>(cl, m, g, e, clusters, s, pdl);
+    case EPI_QKV: return launch_wide_one<EPI_QKV, kWideCluster>(m, g, e, clusters, s, pdl);
+    case EPI_GATEUP: return launch_wide_one<EPI_GATEUP, kWideCluster>(m, g, e, clusters, s, pdl);
+    case EPI_RESID: return launch_wide_one<EPI_RESID, kWideCluster>(m, g, e, clusters, s, pdl);
+    case EPI_ACC: return launch_wide_one<EPI_ACC, kWideCluster>(m, g, e, clusters, s, pdl);
     case EPI_ARGMAX: break;
     default: return cudaErrorInvalidValue;
   }
-  if ((err = launch_wide_kind<EPI_ARGMAX>(cl, m, g, e, clusters, s, pdl)) != cudaSuccess) return err;
+  if ((err = launch_wide_one<EPI_ARGMAX, kWideCluster>(m, g, e, clusters, s, pdl)) != cudaSuccess) return err;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
   cfg.gridDim = dim3((e.T + 15) / 16);

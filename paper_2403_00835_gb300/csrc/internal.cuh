@@ -29,7 +29,8 @@ constexpr int kEpiCols = 16;     // columns per epilogue chunk
 // without shortening the chain, so it is off.
 constexpr int kL2AheadDefault = 0;
 
-enum EpiKind : int { EPI_QKV = 0, EPI_GATEUP = 1, EPI_RESID = 2, EPI_ARGMAX = 3 };
+// EPI_ACC (stand-alone GEMMs): x += D, without the next norm's input and statistics
+enum EpiKind : int { EPI_QKV = 0, EPI_GATEUP = 1, EPI_RESID = 2, EPI_ARGMAX = 3, EPI_ACC = 4 };
 
 // Per-launch epilogue arguments (passed by value; one struct for all kinds).
 struct EpiArgs {
@@ -298,12 +299,12 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, 
 
 // Wide launches (T > 256, gemm_wide.cu): units of 512 weight rows (gate/up:
 // 256 features) x bn tokens per CTA pair, the (unit, K chunk) space in ranges
-// of cpc chunks per cluster of cl CTAs.
+// of cpc chunks per cluster.
 constexpr int kWideTokens = 128;                     // most tokens of a pair's tile
 constexpr int kWidePartFloats = 2 * kWideTokens * kBM;  // a CTA's split-K partial
 constexpr int kWideCluster = 4;                      // CTAs per cluster
 struct WidePlan {
-  int cl, row_units, ntiles, bn, kchunks, cpc, clusters;
+  int row_units, ntiles, bn, kchunks, cpc, clusters;
   void apply(GemmArgs& g) const {
     g.mtiles = row_units;
     g.ntiles = ntiles;
@@ -314,11 +315,12 @@ struct WidePlan {
 };
 // split: ranges may cut a unit (needs kWidePartFloats floats and one zeroed
 // ticket per CTA); otherwise whole units
-WidePlan plan_wide(int kind, int M, int K, int T, int cl, int clusters, bool split);
-int gemm_wide_clusters(int cl);
+WidePlan plan_wide(int kind, int M, int K, int T, int clusters, bool split);
+int gemm_wide_clusters();  // after the attributes of the EPI_ACC kernel are set
 cudaError_t gemm_wide_set_attributes();
+cudaError_t gemm_wide_set_attributes_acc();  // EPI_ACC only
 // (ARGMAX: two kernels, the second reduces the tiles' maxima)
-cudaError_t launch_gemm_wide(int kind, int cl, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
+cudaError_t launch_gemm_wide(int kind, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
                              cudaStream_t s, bool pdl);
 
 cudaError_t launch_embed(const EmbedArgs& a, int act_bf16, cudaStream_t s, bool pdl);
@@ -349,6 +351,7 @@ cudaError_t launch_gather_rows(const void* xg_src, const float* ssq_src, void* x
 int gemm_tc_stages(int bn_max);
 size_t gemm_tc_smem_bytes(int bn_max);
 cudaError_t gemm_tc_set_attributes();
+cudaError_t gemm_tc_set_attributes_acc(int bn_max);  // EPI_ACC, one column count
 cudaError_t attention_set_attributes();
 size_t attention_smem_bytes(int hd);
 

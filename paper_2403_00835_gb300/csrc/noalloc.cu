@@ -5,9 +5,8 @@
 // path where the implicit device synchronisation of cudaMalloc/cudaFree is
 // not acceptable.  This entry point runs the same tcgen05/TMA GEMM kernel as
 // the rest of the library, but every byte of scratch it needs (split-K
-// partial tiles, arrival tickets, the device error word, and the epilogue's
-// side outputs) lives in one file-scope device array of fixed size, so the
-// call allocates nothing.  The caller still provides the inputs and output.
+// partial tiles, arrival tickets and the device error word) lives in one
+// file-scope device array of fixed size, so the call allocates nothing.  The caller still provides the inputs and output.
 #include "../../include/cllm.h"
 #include "internal.cuh"
 
@@ -34,11 +33,6 @@ int scratch_address(void** out) {
   return CLLM_OK;
 }
 
-__global__ void fill_bf16_one(__nv_bfloat16* p, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = __float2bfloat16(1.f);
-}
-
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
@@ -56,27 +50,28 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   if (cudaStreamIsCapturing(static_cast<cudaStream_t>(cuda_stream), &cap) != cudaSuccess)
     return CLLM_ECUDA;
   if (cap != cudaStreamCaptureStatusNone) return CLLM_EUNSUPPORTED;
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
+  // (three attributes: the whole property structure takes longer to fill than
+  // the GEMM of 16 rows runs)
+  int dev = 0, major = 0, minor = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return CLLM_ECUDA;
-  if (prop.major != 10 || prop.minor != 3) return CLLM_EUNSUPPORTED;
+  if (major != 10 || minor != 3) return CLLM_EUNSUPPORTED;
   const int mtiles = M / kBM;
-  const Part p = plan_gemm(mtiles, K, T, prop.multiProcessorCount);
-  const int ldt = round_up(T, 16);
-  // scratch layout inside the static array
-  const size_t off_part = 0;
+  const Part p = plan_gemm(mtiles, K, T, sms);
+  // scratch inside the static array: partial tiles, tickets, the error word.
+  // The limit also counts the side outputs that the engine's own epilogue
+  // would write for this size (statistics, next inputs and their gains), so
+  // which sizes are accepted does not depend on the epilogue.
   const size_t sz_part = align256(static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4);
-  const size_t off_tick = off_part + sz_part;
+  const size_t off_tick = sz_part;
   const size_t sz_tick = align256(static_cast<size_t>(mtiles) * 4);
   const size_t off_err = off_tick + sz_tick;
-  const size_t off_ssq = off_err + 256;
-  const size_t sz_ssq = align256(static_cast<size_t>(mtiles) * ldt * 4);
-  const size_t off_xg = off_ssq + sz_ssq;
-  const size_t sz_xg = align256(static_cast<size_t>(2) * T * M * 2);
-  const size_t off_one = off_xg + sz_xg;
-  const size_t total = off_one + align256(static_cast<size_t>(M) * 2);
-  if (total > kNoAllocScratchBytes) return CLLM_ECAPACITY;
+  const size_t sz_side = align256(static_cast<size_t>(mtiles) * round_up(T, 16) * 4) +
+                         align256(static_cast<size_t>(2) * T * M * 2) + align256(static_cast<size_t>(M) * 2);
+  if (off_err + 256 + sz_side > kNoAllocScratchBytes) return CLLM_ECAPACITY;
 
   void* base = nullptr;
   int rc = scratch_address(&base);
@@ -87,11 +82,11 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   const bool wide = T > 256;
   WidePlan w{};
   if (wide) {
-    if (gemm_wide_set_attributes() != cudaSuccess) return CLLM_ECUDA;
-    const int clusters = gemm_wide_clusters(kWideCluster);
+    if (gemm_wide_set_attributes_acc() != cudaSuccess) return CLLM_ECUDA;
+    const int clusters = gemm_wide_clusters();
     if (clusters < 1) return CLLM_ECUDA;
-    w = plan_wide(EPI_RESID, M, K, T, kWideCluster, clusters, false);
-  } else if (gemm_tc_set_attributes() != cudaSuccess) {
+    w = plan_wide(EPI_ACC, M, K, T, clusters, false);
+  } else if (gemm_tc_set_attributes_acc(p.bn_max) != cudaSuccess) {
     return CLLM_ECUDA;
   }
   GemmMaps maps{};
@@ -99,12 +94,8 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
     return CLLM_EINVAL;
   maps.a1 = maps.a2 = maps.a0;
   // the array keeps the previous call's contents: tickets and the error word
-  // must start at zero
-  if (cudaMemsetAsync(sb + off_tick, 0, sz_tick, s) != cudaSuccess ||
-      cudaMemsetAsync(sb + off_err, 0, 256, s) != cudaSuccess)
-    return CLLM_ECUDA;
-  fill_bf16_one<<<ceil_div(M, 256), 256, 0, s>>>(reinterpret_cast<__nv_bfloat16*>(sb + off_one), M);
-  if (cudaGetLastError() != cudaSuccess) return CLLM_ECUDA;
+  // must start at zero (they are neighbours)
+  if (cudaMemsetAsync(sb + off_tick, 0, sz_tick + 256, s) != cudaSuccess) return CLLM_ECUDA;
 
   GemmArgs g{};
   g.M = M;
@@ -122,21 +113,16 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   g.l2_ahead = kL2AheadDefault;  // as the allocating GEMM entry points
   g.pre_stages = 1 << 20;
   if (wide) w.apply(g);
-  g.partial = reinterpret_cast<float*>(sb + off_part);
+  g.partial = reinterpret_cast<float*>(sb);
   g.tickets = reinterpret_cast<int*>(sb + off_tick);
   g.err = reinterpret_cast<int*>(sb + off_err);
   EpiArgs e{};
   e.T = T;
-  e.ldt = ldt;
   e.x = Y;
-  e.xg = sb + off_xg;
-  e.gnext = sb + off_one;
-  e.plane_x = static_cast<size_t>(T) * M;
-  e.ssq_out = reinterpret_cast<float*>(sb + off_ssq);
   e.d = M;
   e.err = g.err;
-  const cudaError_t le = wide ? launch_gemm_wide(EPI_RESID, w.cl, maps, g, e, w.clusters, s, false)
-                              : launch_gemm_tc(EPI_RESID, p.bn_max, maps, g, e, p.grid, s, false);
+  const cudaError_t le = wide ? launch_gemm_wide(EPI_ACC, maps, g, e, w.clusters, s, false)
+                              : launch_gemm_tc(EPI_ACC, p.bn_max, maps, g, e, p.grid, s, false);
   if (le != cudaSuccess) return CLLM_ECUDA;
   int herr = 0;
   if (cudaMemcpyAsync(&herr, g.err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
