@@ -259,12 +259,16 @@ int cllm_decode_read_stats(cllm_ctx *ctx, cllm_accept_stats *out, int64_t *acc_h
                            int64_t *win_hist);
 
 /* ---- options --------------------------------------------------------------------
- * CLLM_OPT_PERSISTENT (default 1): run each decode/step iteration of the bf16
- * engine as ONE persistent kernel (one CTA per SM; phases embed, per layer
- * QKV / attention / O / gate-up / down, LM head, accept, separated by grid
- * barriers) when B*n <= 128 and head_dim is 64 or 128; 0 = one kernel per
- * phase.  Both paths compute bit-identical results.  Takes effect for graphs
- * captured after the call.  Returns CLLM_OK or EINVAL (unknown option).
+ * CLLM_OPT_PERSISTENT: run a decode/step iteration of the bf16 engine as ONE
+ * persistent kernel (one CTA per SM; phases embed, per layer QKV / attention /
+ * O / gate-up / down, LM head, accept, separated by grid barriers).  Supported
+ * when B*n <= 128 and head_dim is 64 or 128.  1 = wherever it is supported, 0 =
+ * one kernel per phase.  Until the option is set the library takes the
+ * persistent kernel where it is the faster of the two: for blocks of fewer than
+ * 64 rows with at most about one attention item (16 rows of a head against 512
+ * keys) per SM at the sequences' committed lengths.  Both paths compute
+ * bit-identical results.  Takes effect for graphs captured after the call.
+ * Returns CLLM_OK or EINVAL (unknown option).
  */
 #define CLLM_OPT_PERSISTENT 1
 /* CLLM_OPT_PARK_SLOTS (default 0 = all): in the persistent kernel, the weight

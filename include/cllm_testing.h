@@ -93,7 +93,7 @@ int cllm_test_hold_barrier(cllm_ctx *ctx, int phase);
 void cllm_test_fail_alloc(int k);
 
 /*
- * Host-only (no CUDA call): the work split of one weight-GEMM launch of
+ * Host-only (no CUDA call): the work split of a stand-alone weight GEMM of
  * `mtiles` 128-row weight tiles over K (inner dimension) for T token columns
  * on `sms` SMs, as the library plans it.  out[8] = {mtiles, ntiles (token
  * tiles), kchunks (64-column chunks of K), cpc (chunks per CTA), bn (token
@@ -104,6 +104,15 @@ void cllm_test_fail_alloc(int k);
  * or a non-positive argument.
  */
 int cllm_test_plan_gemm(int mtiles, int K, int T, int sms, int *out);
+
+/*
+ * Host-only: the work split of the engine's launches of T <= 256 tokens.
+ * out[8] = {mtiles, tiles per group, kchunks, cpc, bn, bn_max, maxc (most
+ * ranges sharing one tile), grid (CTAs)}.  The tiles form groups of 4; CTA c
+ * works on tile c mod 4 of the groups and on chunks [c/4 * cpc, (c/4 + 1) * cpc)
+ * of that residue's (group, chunk) space.  EINVAL as above, or T > 256.
+ */
+int cllm_test_plan_group(int mtiles, int K, int T, int sms, int *out);
 
 #ifdef __cplusplus
 }

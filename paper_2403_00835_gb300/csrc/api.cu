@@ -57,7 +57,7 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, 
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Split of one GEMM launch over the SMs.  T <= 256: one N-tile holding every
+// Split of one stand-alone GEMM over the SMs.  T <= 256: one N-tile holding every
 // token and the (tile, k-chunk) space cut into equal contiguous ranges; the
 // cut depends on the weight shape and the SM count only.  T > 256: whole
 // 128 x 256 tiles per CTA, no split.  Chunks per tile and per CTA are even,
@@ -91,6 +91,35 @@ Part plan_gemm(int mtiles, int K, int T, int sms) {
     p.grid = ceil_div(units, upc);
     p.maxc = 1;
   }
+  return p;
+}
+
+// Split of the engine's launches of up to 256 tokens: groups of 4 tiles whose
+// (group, k-chunk) space is cut into sms / 4 ranges, each worked on by 4 CTAs,
+// one tile of the group each.  Neighbouring CTAs then run over the same K
+// range at the same time, which is what lets a CTA pair share its activation
+// tiles; the share of each CTA is that of plan_gemm's split (7B QKV 42 chunks,
+// O 14, gate/up 74, down 38 of 152 CTAs either way).  Like there, the cut
+// depends on the weight shape and the SM count only, and ranges and tiles
+// start on a pair of chunks.  A range has at least kMinRange chunks: below
+// that the exchange of partial sums takes longer than the chunks (a small
+// decoder's phase).
+constexpr int kMinRange = 4;
+
+Part plan_group(int mtiles, int K, int T, int sms) {
+  Part p{};
+  const int size = 1 << kGroupShift;
+  p.mtiles = mtiles;
+  p.ntiles = 1;
+  p.kchunks = round_up(ceil_div(K, kBK), 2);
+  p.bn = round_up(std::max(T, 1), 16);
+  p.bn_max = p.bn <= 32 ? 32 : (p.bn <= 64 ? 64 : (p.bn <= 128 ? 128 : 256));
+  const int groups = ceil_div(mtiles, size), C = groups * p.kchunks;
+  p.cpc = std::max(kMinRange, round_up(ceil_div(C, std::max(1, sms / size)), 2));
+  p.grid = size * ceil_div(C, p.cpc);
+  p.maxc = 1;
+  for (int u = 0; u < groups; ++u)
+    p.maxc = std::max(p.maxc, ((u + 1) * p.kchunks - 1) / p.cpc - (u * p.kchunks) / p.cpc + 1);
   return p;
 }
 
@@ -195,7 +224,9 @@ struct cllm_ctx {
     unsigned long long* cta_stamps = nullptr;
     size_t bar_bytes = 64;             // grid-barrier counter and completion flags
   };
-  bool persistent = true;  // one persistent kernel per iteration where supported
+  // one persistent kernel per iteration: -1 where it is faster, 1 wherever it is
+  // supported, 0 never
+  int persistent = -1;
   int park_slots = 0;  // persistent kernel: tensor-memory park slots in use (0: all)
   int l2_pairs = 0;    // persistent kernel: weight pairs prefetched into L2 when the ring is full
   bool dataflow = true;  // persistent kernel: attention and O open on completion flags
@@ -307,7 +338,8 @@ GemmArgs tc_gemm_args(cllm_ctx* c, int mtiles, int M, int K, int T, EpiArgs& e, 
   g.lo_rows = c->Tcap;
   g.l2_ahead = kL2AheadDefault;
   g.pre_stages = 1 << 20;
-  const Part p = plan_gemm(mtiles, K, T, c->sms);
+  const Part p = plan_group(mtiles, K, T, c->sms);
+  g.gshift = kGroupShift;
   g.mtiles = p.mtiles;
   g.ntiles = p.ntiles;
   g.kchunks = p.kchunks;
@@ -367,16 +399,16 @@ cudaError_t gemm(cllm_ctx* c, cudaStream_t s, bool pdl, int kind, int mtiles, in
     }
     Part p;
     g = tc_gemm_args(c, mtiles, M, K, T, ee, &p);
-    if (static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM > c->gemm_part_elems && p.ntiles == 1)
+    if (static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM > c->gemm_part_elems)
       return cudaErrorInvalidValue;
     GemmMaps maps{};
     maps.a0 = *m0;
     maps.a1 = m1 ? *m1 : *m0;
     maps.a2 = m2 ? *m2 : *m0;
     if (!make_map(&maps.b, X, static_cast<uint64_t>(K), static_cast<uint64_t>(2 * c->Tcap),
-                  static_cast<uint32_t>(p.bn)))
+                  static_cast<uint32_t>(pair_box_rows(p.bn))))
       return cudaErrorInvalidValue;
-    err = launch_gemm_tc(kind, p.bn_max, maps, g, ee, p.grid, s, pdl);
+    err = launch_gemm_pair(kind, maps, g, ee, p.grid, s, pdl);
   }
   return after_launch(c, s, name, err);
 }
@@ -739,7 +771,6 @@ int build_persistent(cllm_ctx* c, int mode, int B, int n, const int2* qtiles, in
     unsigned* head_done = qkv_done + Mqkv / kBM;
     if (c->dataflow) e.tile_done = qkv_done;
     gemm_phase(EPI_QKV, 7 * l, 7 * l + 1, 7 * l + 2, mapB, Mqkv / kBM, Mqkv, c->d, e);
-    const int qkv_ntiles = ph.back().g.ntiles;
     PhaseDesc at{};
     at.kind = PH_ATTN;
     at.k_cache = kl;
@@ -749,7 +780,7 @@ int build_persistent(cllm_ctx* c, int mode, int B, int n, const int2* qtiles, in
       at.no_barrier = 1;
       at.qkv_done = qkv_done;
       at.head_done = head_done;
-      at.flag_target = qkv_ntiles;
+      at.flag_target = 1;
     }
     ph.push_back(at);
     e = base_epi(c, T);
@@ -856,11 +887,28 @@ int build_persistent(cllm_ctx* c, int mode, int B, int n, const int2* qtiles, in
   return CLLM_OK;
 }
 
+// Whether an iteration of B x n rows runs as the persistent kernel: where it is
+// supported and, unless the caller has chosen, faster than one kernel per
+// phase on CTA pairs.  (Both give the same bits.)  7B shape, 8 layers, us per iteration, persistent against pairs:
+// the pairs fetch less activation data per weight tile, which decides from 64
+// rows on (64 rows 1081 / 1061, 96 1440 / 1169, 128 1692 / 1269; 48 rows 983 /
+// 1031); below that the persistent kernel saves the launches, until its one
+// CTA per SM has more than about a wave of attention items of up to 512 keys
+// (16 rows at 2048 keys, 160 items: 926 / 969; at 4096, 288: 1053 / 1017; 32
+// rows at 512 keys, 128: 951 / 973; at 1024, 192: 1033 / 981; 8 sequences at
+// 1024 keys, 768: 1300 / 1131).
 bool persistent_ok(cllm_ctx* c, int B, int n) {
   // (the attention's K/V tensor maps address cache rows with 32-bit coordinates)
-  return c->bf16 && c->persistent && B * n <= 128 && 7 * c->NL + 7 <= kMaxStepMaps &&
-         static_cast<uint64_t>(c->NL) * c->layer_kv_elems / c->hd + kAttnChunk < (1ull << 31) &&
-         B * ceil_div(n, kQTile) <= kMaxQTilesStep && (c->hd == 64 || c->hd == 128);
+  if (!(c->bf16 && c->persistent != 0 && B * n <= 128 && 7 * c->NL + 7 <= kMaxStepMaps &&
+        static_cast<uint64_t>(c->NL) * c->layer_kv_elems / c->hd + kAttnChunk < (1ull << 31) &&
+        B * ceil_div(n, kQTile) <= kMaxQTilesStep && (c->hd == 64 || c->hd == 128)))
+    return false;
+  if (c->persistent == 1) return true;
+  if (B * n >= 64) return false;
+  long items = 0;
+  for (int b = 0; b < B; ++b)
+    items += static_cast<long>(c->H) * ceil_div(n, kQTile) * ceil_div(c->Lh[b] + n, kAttnChunk * kAttnRange);
+  return items <= c->sms + c->sms / 8;
 }
 
 // Get (capturing on first use) the graph of one decode/step iteration.
@@ -875,7 +923,7 @@ int get_graph(cllm_ctx* c, int mode, int n, cllm_ctx::GraphEntry** out) {
                              (c->profiling ? 1 : 0) | (mode == MODE_STEP && c->step_logits ? 2 : 0) |
                                  (mode == MODE_DECODE && c->dec_opts.stats ? 4 : 0) |
                                  (mode == MODE_DECODE ? (c->dec_opts.ngram << 3) : 0),
-                             c->persistent ? 1 : 0,
+                             persistent_ok(c, B, n) ? 1 : 0,
                              (c->park_slots * 4096 + c->l2_pairs) * 2 + (c->dataflow ? 1 : 0));
   auto it = c->graphs.find(key);
   if (it != c->graphs.end()) {
@@ -1228,9 +1276,9 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
         rc = CLLM_EINVAL;
         break;
       }
-      if (gemm_tc_set_attributes() != cudaSuccess || attention_set_attributes() != cudaSuccess ||
+      if (attention_set_attributes() != cudaSuccess ||
           step_persistent_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess ||
-          gemm_wide_set_attributes_acc() != cudaSuccess ||
+          gemm_wide_set_attributes_acc() != cudaSuccess || gemm_pair_set_attributes() != cudaSuccess ||
           attention_wide_set_attributes() != cudaSuccess) {
         rc = CLLM_ECUDA;
         break;
@@ -1312,7 +1360,7 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
     size_t need = 0;
     c->max_mtiles = 0;
     for (int i = 0; i < 5; ++i) {
-      const Part p = plan_gemm(mt_list[i], k_list[i], std::min(256, bn_split), c->sms);
+      const Part p = plan_group(mt_list[i], k_list[i], std::min(256, bn_split), c->sms);
       need = std::max(need, static_cast<size_t>(mt_list[i]) * p.maxc * p.bn * kBM);
       c->max_mtiles = std::max(c->max_mtiles, mt_list[i]);
     }
@@ -1796,7 +1844,7 @@ extern "C" int cllm_ar_decode(cllm_ctx* c, int B, const int32_t* tokens, const i
 extern "C" int cllm_set_option(cllm_ctx* c, int option, int value) {
   if (!c) return CLLM_EINVAL;
   if (option == CLLM_OPT_PERSISTENT) {
-    c->persistent = value != 0;
+    c->persistent = value != 0 ? 1 : 0;
     return CLLM_OK;
   }
   if (option == CLLM_OPT_L2_PAIRS) {
@@ -2128,6 +2176,14 @@ extern "C" int cllm_test_plan_gemm(int mtiles, int K, int T, int sms, int* out) 
   const Part p = plan_gemm(mtiles, K, T, sms);
   const int v[8] = {p.mtiles, p.ntiles, p.kchunks, p.cpc, p.bn, p.bn_max, p.maxc, p.grid};
   for (int i = 0; i < 8; ++i) out[i] = v[i];
+  return CLLM_OK;
+}
+
+extern "C" int cllm_test_plan_group(int mtiles, int K, int T, int sms, int* out) {
+  if (!out || mtiles < 1 || K < 1 || T < 1 || T > 256 || sms < 1) return CLLM_EINVAL;
+  const Part p = plan_group(mtiles, K, T, sms);
+  const int v[8] = {p.mtiles, 1 << kGroupShift, p.kchunks, p.cpc, p.bn, p.bn_max, p.maxc, p.grid};
+  std::memcpy(out, v, sizeof v);
   return CLLM_OK;
 }
 

@@ -10,9 +10,8 @@
 // memory (128 columns), a thread per row turns its 128 scores into fp16
 // probabilities written back over S, and P V accumulates with P read from
 // tensor memory (A operand) and V from shared memory (MN-major B operand).
-// The running maximum is only moved when a row's maximum has grown by more
-// than 2^8 (probabilities are then at most 256, sums stay fp32), so the output
-// accumulator is rescaled rarely.  One thread issues every TMA load and MMA:
+// The output accumulator is rescaled when a row's running maximum has grown,
+// which a warp votes on, so chunks after the first few rarely pay for it.  One thread issues every TMA load and MMA:
 // the order of its waits also tells it when a K or V buffer is free.
 //
 // Compute: 2 x 128 x 128 x hd x 2 FLOP per tile and chunk, 0.26 us per MMA
@@ -36,7 +35,6 @@ constexpr int kWAttnThreads = 256 + 128;
 constexpr int kWAttnRegsLow = 56, kWAttnRegsRow = 224;
 static_assert(128 * kWAttnRegsLow + 256 * kWAttnRegsRow <= kWAttnThreads * 168, "register split");
 constexpr int kWQ = 128;                 // query rows per tile
-constexpr float kRescaleLog2 = 8.f;
 
 template <int HD>
 struct WideAttnSmem {
@@ -221,7 +219,7 @@ __global__ void __launch_bounds__(kWAttnThreads, 1)
         for (int u = 0; u < 4; ++u) m4[u] = fmaxf(m4[u], fmaxf(x0[i + u], x1[i + u]));
       const float cm = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * a.scale_log2;
       // (chunk 0 holds position 0, which every row sees)
-      const bool grow = cm > mx + kRescaleLog2;
+      const bool grow = cm > mx;
       if (c == 0) {
         mx = cm;
       } else if (__any_sync(0xffffffffu, grow)) {

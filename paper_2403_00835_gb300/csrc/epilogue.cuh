@@ -56,6 +56,12 @@ __device__ __forceinline__ void epi_sync() { named_bar_sync(1, 128); }
 // column is in flight at once; the order does not depend on the launch).
 // Sum of column t's per-tile squares by the 8 threads part = 0..7 (tiles
 // part, part + 8, ... in order) followed by a fixed shuffle tree.
+__device__ __forceinline__ float epi_ssq_tree(float acc) {
+  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+  return acc;
+}
 __device__ __forceinline__ float epi_ssq_column(const EpiArgs& e, int t, int part, bool valid) {
   float acc = 0.f;
   if (valid) {
@@ -69,27 +75,58 @@ __device__ __forceinline__ float epi_ssq_column(const EpiArgs& e, int t, int par
     for (int u = 0; u < 8; ++u) acc += v[u];
     for (int i = part + 64; i < e.ssq_tiles; i += 8) acc += __ldcg(e.ssq_in + static_cast<size_t>(i) * e.ldt + t);
   }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-  return acc;
+  return epi_ssq_tree(acc);
+}
+
+// The same sums for columns t .. t + 3 (t a multiple of 4, inside the launch's
+// padded columns), a quarter of the requests: every CTA of a launch reads the
+// same few lines, and at 256 columns the requests for single floats kept the
+// L2 busy for 10 us.
+__device__ __forceinline__ void epi_ssq_quad(const EpiArgs& e, int t, int part, float (&acc)[4]) {
+  const float4* p = reinterpret_cast<const float4*>(e.ssq_in + t);
+  const size_t ld = static_cast<size_t>(e.ldt) / 4;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) acc[c] = 0.f;
+  for (int i0 = part; i0 < e.ssq_tiles; i0 += 32) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      v[u] = i0 + 8 * u < e.ssq_tiles ? __ldcg(p + (i0 + 8 * u) * ld) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      acc[0] += v[u].x;
+      acc[1] += v[u].y;
+      acc[2] += v[u].z;
+      acc[3] += v[u].w;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) acc[c] = epi_ssq_tree(acc[c]);
 }
 
 // Once per launch / phase, before the first accumulator is ready: the RMSNorm
-// scale (kinds that need it), position and sequence index of every column.
+// scale (kinds that need it), position and sequence index of the columns of
+// the 16-column chunks gi, gi + ng, ... (those of this group of threads).
 template <int KIND>
-__device__ void epi_prepare(const EpiArgs& e, int r, EpiSmem& s) {
+__device__ void epi_prepare(const EpiArgs& e, int r, EpiSmem& s, int gi = 0, int ng = 1) {
   s.prepared = 0;
   if (e.T > kEpiPrepMax) {
     epi_sync();
     return;
   }
   if (KIND != EPI_RESID && KIND != EPI_ACC) {
-    const int col = r >> 3, part = r & 7;
-    for (int t0 = 0; t0 < e.T; t0 += kEpiCols) {
-      const int t = t0 + col;
-      const float acc = epi_ssq_column(e, t, part, t < e.T);
-      if (part == 0 && t < e.T) s.rs_all[t] = rsqrtf(acc * e.inv_d + e.eps);
+    const int quad = r >> 3, part = r & 7;  // 16 column quads (4 chunks) at a time
+    const int nch = (e.T + kEpiCols - 1) / kEpiCols;
+    for (int c0 = gi; c0 < nch; c0 += 4 * ng) {
+      const int ch = c0 + (quad >> 2) * ng;
+      if (c0 + ((r & ~31) >> 5) * ng >= nch) continue;  // (a warp's 4 quads are one chunk)
+      const int t = ch * kEpiCols + (quad & 3) * 4;
+      float ss[4];
+      epi_ssq_quad(e, t, part, ss);
+      if (part < 4 && t + part < e.T) {
+        const float v = part == 0 ? ss[0] : part == 1 ? ss[1] : part == 2 ? ss[2] : ss[3];
+        s.rs_all[t + part] = rsqrtf(v * e.inv_d + e.eps);
+      }
     }
   }
   if (KIND == EPI_QKV) {
@@ -293,23 +330,31 @@ __device__ void epi_apply(const EpiArgs& e, int mt, int t0, float (&v)[kEpiCols]
       s.x[j][r] = v[j];
     }
     epi_sync();
-    if (r < 64) {
-      const int f = mt * 64 + r;
-      if (f < e.F) {
-        float h[kEpiCols];  // SwiGLU of every column first, then the stores
+    // both halves of the tile's threads work: gate rows on columns 0-7, up rows
+    // on columns 8-15 of the same features
+    const bool low = r < 64;
+    const int f = mt * 64 + (r & 63);
+    if (f < e.F) {
+      constexpr int HC = kEpiCols / 2;
+      const int jb = low ? 0 : HC;
+      float gt[HC], up[HC], h[HC];  // SwiGLU of every column first, then the stores
 #pragma unroll
-        for (int j = 0; j < kEpiCols; ++j) {
-          const float gt = v[j], up = s.x[j][r + 64];
-          if constexpr (std::is_same<Act, float>::value)
-            h[j] = gt / (1.f + expf(-gt)) * up;
-          else  // bf16 engine: the fast intrinsics' error is far below the lo plane's
-            h[j] = __fdividef(gt, 1.f + __expf(-gt)) * up;
-        }
-        Act* hp = reinterpret_cast<Act*>(e.h_out) + static_cast<size_t>(t0) * e.F + f;
-#pragma unroll
-        for (int j = 0; j < kEpiCols; ++j)
-          if (full || t0 + j < e.T) st_gin(hp, static_cast<size_t>(j) * e.F, e.plane_h, h[j]);
+      for (int j = 0; j < HC; ++j) {
+        const float other = s.x[jb + j][r ^ 64];
+        gt[j] = low ? v[j] : other;
+        up[j] = low ? other : v[HC + j];
       }
+#pragma unroll
+      for (int j = 0; j < HC; ++j) {
+        if constexpr (std::is_same<Act, float>::value)
+          h[j] = gt[j] / (1.f + expf(-gt[j])) * up[j];
+        else  // bf16 engine: the fast intrinsics' error is far below the lo plane's
+          h[j] = __fdividef(gt[j], 1.f + __expf(-gt[j])) * up[j];
+      }
+      Act* hp = reinterpret_cast<Act*>(e.h_out) + static_cast<size_t>(t0 + jb) * e.F + f;
+#pragma unroll
+      for (int j = 0; j < HC; ++j)
+        if (full || t0 + jb + j < e.T) st_gin(hp, static_cast<size_t>(j) * e.F, e.plane_h, h[j]);
     }
     epi_sync();
   } else if (KIND == EPI_ACC) {

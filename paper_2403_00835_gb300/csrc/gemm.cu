@@ -1,27 +1,20 @@
-// Weight-streaming GEMMs of the block forward, with fused epilogues.
+// The weight-streaming GEMM on its own (the allocation-free entry point and the
+// test hooks; the engine's launches run on CTA pairs, gemm_pair.cu and
+// gemm_wide.cu, or inside the persistent kernel).
 //
 //   D[m][t] = sum_k W[m][k] * X[t][k]      (W: [M][K] weights, X: [T][K] activations)
 //
-// At the small token counts of a Jacobi step (T = batch * n <= 256) every
-// weight byte is used T times, so the GEMMs are bound by streaming W from
-// HBM.  The bf16 kernel is "swap-AB": the weight tile is the MMA's A operand
-// (M = 128 rows), the tokens are its N (16..256 columns), and the fp32
-// accumulator lives in tensor memory (TMEM).  A producer warp streams W and X
-// tiles with TMA into a ring of shared-memory stages, one thread issues
-// tcgen05.mma, and four epilogue warps read TMEM.  The grid is one CTA per SM;
-// the (tile, k-chunk) space is cut into equal contiguous ranges, so a tile
-// whose K range is split over several CTAs is finished by the last one to
-// arrive (atomic ticket, no waiting), which sums the partial tiles in a fixed
-// order.  The partition depends only on the weight shape and SM count, never
-// on T, so a token's result does not depend on how many rows share the launch.
-//
-// Fused epilogues (each reads the RMSNorm statistics its producer left):
-//   EPI_QKV    : x rms-scale, rotate-half RoPE, Q -> scratch, K/V -> cache
-//   EPI_GATEUP : x rms-scale, silu(gate) * up -> h
-//   EPI_RESID  : residual add into the fp32 stream, next norm's input and
-//                per-tile sum of squares
-//   EPI_ARGMAX : x rms-scale, per-tile (max, argmax, 2nd max) of the logits;
-//                the last tile to finish reduces them to argmax and top-2 gap
+// At small token counts every weight byte is used T times, so the GEMM is
+// bound by streaming W from HBM.  The kernel is "swap-AB": the weight tile is
+// the MMA's A operand (M = 128 rows), the tokens are its N (16..256 columns),
+// and the fp32 accumulator lives in tensor memory (TMEM).  A producer warp
+// streams W and X tiles with TMA into a ring of shared-memory stages, one
+// thread issues tcgen05.mma, and four epilogue warps read TMEM.  The grid is
+// one CTA per SM; the (tile, k-chunk) space is cut into equal contiguous
+// ranges, and a tile whose K range is split over several CTAs is reduced by
+// its first contributor in a fixed order.  The partition depends only on the
+// weight shape and SM count, never on T, so a token's result does not depend
+// on how many rows share the launch.
 #include <float.h>
 #include <limits.h>
 
@@ -98,7 +91,7 @@ __global__ void __launch_bounds__(64 + 128 * solo_groups<KIND, BNMAX>(), 1)
   if (warp == 0) {
     if (lane == 0) {
       int idx = 0, issued = 0;
-      tc_produce<KIND, Cfg>(P, idx, issued, g, &mA0, &mA1, &mA2, &mB, c0, c1, PdlDep{});
+      tc_produce<KIND, Cfg>(P, idx, issued, g, &mA0, &mA1, &mA2, &mB, c0, c1, blockIdx.x, PdlDep{});
       tc_produce_drain<Cfg>(P, issued);
     }
   } else if (warp == 1) {
@@ -127,24 +120,6 @@ __global__ void __launch_bounds__(64 + 128 * solo_groups<KIND, BNMAX>(), 1)
 // launchers
 // ---------------------------------------------------------------------------------
 
-int gemm_tc_stages(int bn_max) {
-  switch (bn_max) {
-    case 32: return SoloCfg<32>::STAGES;
-    case 64: return SoloCfg<64>::STAGES;
-    case 128: return SoloCfg<128>::STAGES;
-    default: return SoloCfg<256>::STAGES;
-  }
-}
-
-size_t gemm_tc_smem_bytes(int bn_max) {
-  switch (bn_max) {
-    case 32: return solo_smem_bytes<32>();
-    case 64: return solo_smem_bytes<64>();
-    case 128: return solo_smem_bytes<128>();
-    default: return solo_smem_bytes<256>();
-  }
-}
-
 template <int KIND, int BN>
 static cudaError_t set_attr_one() {
   cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<KIND, BN>,
@@ -156,21 +131,12 @@ static cudaError_t set_attr_one() {
                               static_cast<int>(cudaSharedmemCarveoutMaxShared));
 }
 
-template <int KIND>
-static cudaError_t set_attr_kind() {
-  cudaError_t err;
-  if ((err = set_attr_one<KIND, 32>()) != cudaSuccess) return err;
-  if ((err = set_attr_one<KIND, 64>()) != cudaSuccess) return err;
-  if ((err = set_attr_one<KIND, 128>()) != cudaSuccess) return err;
-  return set_attr_one<KIND, 256>();
-}
-
 cudaError_t gemm_tc_set_attributes() {
   cudaError_t err;
-  if ((err = set_attr_kind<EPI_QKV>()) != cudaSuccess) return err;
-  if ((err = set_attr_kind<EPI_GATEUP>()) != cudaSuccess) return err;
-  if ((err = set_attr_kind<EPI_RESID>()) != cudaSuccess) return err;
-  return set_attr_kind<EPI_ARGMAX>();
+  if ((err = set_attr_one<EPI_RESID, 32>()) != cudaSuccess) return err;
+  if ((err = set_attr_one<EPI_RESID, 64>()) != cudaSuccess) return err;
+  if ((err = set_attr_one<EPI_RESID, 128>()) != cudaSuccess) return err;
+  return set_attr_one<EPI_RESID, 256>();
 }
 
 cudaError_t gemm_tc_set_attributes_acc(int bn_max) {
@@ -219,10 +185,7 @@ static cudaError_t launch_tc_kind(int bn_max, const GemmMaps& m, const GemmArgs&
 cudaError_t launch_gemm_tc(int kind, int bn_max, const GemmMaps& maps, const GemmArgs& g,
                            const EpiArgs& e, int grid, cudaStream_t s, bool pdl) {
   switch (kind) {
-    case EPI_QKV: return launch_tc_kind<EPI_QKV>(bn_max, maps, g, e, grid, s, pdl);
-    case EPI_GATEUP: return launch_tc_kind<EPI_GATEUP>(bn_max, maps, g, e, grid, s, pdl);
     case EPI_RESID: return launch_tc_kind<EPI_RESID>(bn_max, maps, g, e, grid, s, pdl);
-    case EPI_ARGMAX: return launch_tc_kind<EPI_ARGMAX>(bn_max, maps, g, e, grid, s, pdl);
     case EPI_ACC: return launch_tc_kind<EPI_ACC>(bn_max, maps, g, e, grid, s, pdl);
     default: return cudaErrorInvalidValue;
   }

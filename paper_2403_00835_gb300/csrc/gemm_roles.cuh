@@ -52,6 +52,10 @@ struct TcPipe {
   float* red;
   int red_slots;
   int* jflag;  // two epilogue groups, shared memory: [0] the split-K wait's result, [1] the accumulator wait's
+  // CTA pairs
+  uint32_t tempty_leader;  // address of the even CTA's tempty
+  uint8_t* ring_free;      // the stage ring, idle once the last segment's MMAs are done
+  uint64_t* part_bar;      // [groups][kPartRounds]
 };
 
 constexpr size_t kRedSlotBytes = sizeof(float) * kEpiCols * kBM;
@@ -163,7 +167,17 @@ struct Segment {
   int unit, k0, k1;
 };
 
-// Iterate the (unit, k-range) segments of the chunk range [c, c1).
+// Work split of a launch.  The weight rows' 128-row tiles form groups of
+// 1 << g.gshift tiles, and CTA `cta` works on tile `cta mod group size` of the
+// groups: CTAs of one residue share a (group, k-chunk) space cut into equal
+// contiguous ranges of g.cpc chunks, range cta >> gshift to this CTA.  (gshift
+// 0: every tile is a group.  With 4 tiles a group, four neighbouring CTAs
+// always work on the same K range, so a pair of them can share activations.)
+__device__ __forceinline__ int tile_of(const GemmArgs& g, int group, int cta) {
+  return (group << g.gshift) + (cta & ((1 << g.gshift) - 1));
+}
+
+// Iterate the (group, k-range) segments of the chunk range [c, c1).
 __device__ __forceinline__ bool next_segment(int& c, int c1, int kchunks, Segment& sg) {
   if (c >= c1) return false;
   sg.unit = c / kchunks;
@@ -174,10 +188,11 @@ __device__ __forceinline__ bool next_segment(int& c, int c1, int kchunks, Segmen
   return true;
 }
 
-// Chunk range of CTA `cta` in a launch's work split.
+// Chunk range of CTA `cta` (up to the last group that has its tile).
 __device__ __forceinline__ void cta_range(const GemmArgs& g, int cta, int& c0, int& c1) {
-  const int total = g.mtiles * g.ntiles * g.kchunks;
-  c0 = min(total, cta * g.cpc);
+  const int size = 1 << g.gshift;
+  const int total = ((g.mtiles - (cta & (size - 1)) + size - 1) >> g.gshift) * g.kchunks;
+  c0 = min(total, (cta >> g.gshift) * g.cpc);
   c1 = min(total, c0 + g.cpc);
 }
 
@@ -188,7 +203,7 @@ __device__ __forceinline__ void cta_range(const GemmArgs& g, int cta, int& c0, i
 template <int KIND, class Cfg, class Dep>
 __device__ bool tc_produce(const TcPipe& P, int& idx, int& issued_b, const GemmArgs& g,
                            const CUtensorMap* mA0, const CUtensorMap* mA1, const CUtensorMap* mA2,
-                           const CUtensorMap* mB, int c0, int c1, const Dep& dep) {
+                           const CUtensorMap* mB, int c0, int c1, int cta, const Dep& dep) {
   constexpr int S = Cfg::STAGES;
   const int n = c1 - c0;
   if (n <= 0) {
@@ -197,12 +212,11 @@ __device__ bool tc_produce(const TcPipe& P, int& idx, int& issued_b, const GemmA
   }
   const uint64_t pol_w = l2_policy_evict_first();
   const uint64_t pol_x = l2_policy_evict_last();
-  const bool tile_mode = g.ntiles > 1;
   const uint32_t b_bytes = 2u * static_cast<uint32_t>(g.bn) * kBK * 2;
   auto load_a = [&](int j, int st) {
     const int c = c0 + j;
     const int u = c / g.kchunks, k = c - u * g.kchunks;
-    const int mt = u / g.ntiles;
+    const int mt = tile_of(g, u, cta);
     uint8_t* dst = P.sA + st * Cfg::A_BYTES;
     if (KIND == EPI_GATEUP) {
       tma_load_2d(dst, mA0, &P.full[st], k * kBK, mt * 64, pol_w);
@@ -221,18 +235,16 @@ __device__ bool tc_produce(const TcPipe& P, int& idx, int& issued_b, const GemmA
   };
   auto load_b = [&](int j, int st) {
     const int c = c0 + j;
-    const int u = c / g.kchunks, k = c - u * g.kchunks;
-    const int nt = u % g.ntiles;
-    const int row0 = tile_mode ? nt * Cfg::BN : 0;
+    const int k = c % g.kchunks;
     uint8_t* dst = P.sB + st * Cfg::B_BYTES;
-    tma_load_2d(dst, mB, &P.full[st], k * kBK, row0, pol_x);
-    tma_load_2d(dst + (Cfg::STACKED ? g.bn * kBK * 2 : Cfg::B_HALF), mB, &P.full[st], k * kBK,
-                g.lo_rows + row0, pol_x);
+    tma_load_2d(dst, mB, &P.full[st], k * kBK, 0, pol_x);
+    tma_load_2d(dst + (Cfg::STACKED ? g.bn * kBK * 2 : Cfg::B_HALF), mB, &P.full[st], k * kBK, g.lo_rows,
+                pol_x);
   };
   auto prefetch_l2 = [&](int j) {
     const int c = c0 + j;
     const int u = c / g.kchunks, k = c - u * g.kchunks;
-    const int mt = u / g.ntiles;
+    const int mt = tile_of(g, u, cta);
     if (KIND == EPI_GATEUP) {
       tma_prefetch_l2_2d(mA0, k * kBK, mt * 64);
       tma_prefetch_l2_2d(mA1, k * kBK, mt * 64);
@@ -406,6 +418,28 @@ __device__ __forceinline__ void tmem_ld_sum_cfg(uint32_t taddr, int ch, int bn, 
   for (int j = 0; j < kEpiCols; ++j) v[j] += vlo[j];
 }
 
+// Split-K partials of the CTA-pair kernels: 16 columns of row r of chunk ch as
+// four 16-byte pieces, a piece of the 128 rows contiguous.
+__device__ __forceinline__ void part_st16(float* part, int ch, int r, const float (&v)[kEpiCols]) {
+  float4* p = reinterpret_cast<float4*>(part) + static_cast<size_t>(ch) * 4 * kBM + r;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) __stcg(p + q * kBM, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+}
+// (from a copy of the chunk in shared memory)
+__device__ __forceinline__ void part_add16(float (&v)[kEpiCols], const uint8_t* chunk, int r) {
+  const float4* p = reinterpret_cast<const float4*>(chunk) + r;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float4 t = p[q * kBM];
+    v[4 * q] += t.x;
+    v[4 * q + 1] += t.y;
+    v[4 * q + 2] += t.z;
+    v[4 * q + 3] += t.w;
+  }
+}
+constexpr int kPartChunkBytes = kEpiCols * kBM * 4;
+constexpr int kPartRounds = 3;  // rounds of four chunks in flight per epilogue group
+
 // Persistent kernel: publish a finished output tile (its stores are read next
 // by other CTAs, some through TMA) on its completion flag.
 __device__ __forceinline__ void epi_publish(const EpiArgs& e, int mt, int r) {
@@ -420,7 +454,9 @@ __device__ __forceinline__ void epi_publish(const EpiArgs& e, int mt, int r) {
 // slots) take alternate 16-column chunks of each unit; a barrier over both
 // groups orders their stores before the split-K release, the ticket reset
 // and the argmax reduction.  Per column the arithmetic is unchanged.
-template <int KIND, class Cfg, int NG = 1>
+// PAIR: the accumulators belong to a CTA pair, whose even CTA issues the MMAs;
+// a CTA whose tile lies past the last one only hands its accumulator back.
+template <int KIND, class Cfg, int NG = 1, bool PAIR = false>
 __device__ bool tc_epilogue(const TcPipe& P, int& acc, uint32_t& accph, const GemmArgs& g,
                             const EpiArgs& e, int c0, int c1, int cta, EpiSmem& es) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -431,15 +467,25 @@ __device__ bool tc_epilogue(const TcPipe& P, int& acc, uint32_t& accph, const Ge
     if constexpr (NG > 1) named_bar_sync(3, 128 * NG);
     else epi_sync();
   };
-  const bool tile_mode = g.ntiles > 1;
-  if (c0 < c1) epi_prepare<KIND>(e, r, es);
+  auto release = [&]() {  // this warp is done with the accumulator
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+      if constexpr (PAIR) mbar_arrive_remote(P.tempty_leader + 8u * acc);
+      else mbar_arrive(&P.tempty[acc]);
+    }
+  };
+  if (c0 < c1) epi_prepare<KIND>(e, r, es, gi, NG);
   int c = c0;
   Segment sg;
   while (next_segment(c, c1, g.kchunks, sg)) {
-    const int u = sg.unit;
-    const int mt = u / g.ntiles, nt = u - mt * g.ntiles;
+    const int mt = tile_of(g, sg.unit, cta);
     EpiPre pre;
-    epi_prefetch<KIND, __nv_bfloat16>(e, mt, (tile_mode ? nt * Cfg::BN : 0) + gi * kEpiCols, r, es, pre);
+    const bool past = PAIR && mt >= g.mtiles;
+    // (pairs, QKV: the tile's RoPE rows stay in L1, and its registers are needed)
+    constexpr bool kPre = !(PAIR && KIND == EPI_QKV);
+    const EpiPre* use_pre = kPre ? &pre : nullptr;
+    if (kPre && !past) epi_prefetch<KIND, __nv_bfloat16>(e, mt, gi * kEpiCols, r, es, pre);
     bool seg_ok;
     if constexpr (NG > 1) {
       // one wait for both groups: a group that returned alone would leave the
@@ -458,18 +504,24 @@ __device__ bool tc_epilogue(const TcPipe& P, int& acc, uint32_t& accph, const Ge
     const bool dbg = e.dbg != nullptr && r == 0 && c >= c1;  // last segment
     if (dbg) e.dbg[cta] = globaltimer_ns();
     tc_fence_after();
-    const int first = (u * g.kchunks) / g.cpc;
-    const int last = ((u + 1) * g.kchunks - 1) / g.cpc;
+    if (past) {
+      release();
+      if (++acc == Cfg::NACC) {
+        acc = 0;
+        accph ^= 1;
+      }
+      continue;
+    }
+    const int first = (sg.unit * g.kchunks) / g.cpc;
+    const int last = ((sg.unit + 1) * g.kchunks - 1) / g.cpc;
     const int nc = last - first + 1;
-    const int slot = cta - first;
-    const int tbase = tile_mode ? nt * Cfg::BN : 0;
-    const int ncols = min(g.bn, e.T - tbase);
-    const int nchunk = (ncols + kEpiCols - 1) / kEpiCols;
+    const int slot = (cta >> g.gshift) - first;
+    const int nchunk = (e.T + kEpiCols - 1) / kEpiCols;
     const uint32_t taddr = P.tmem + (static_cast<uint32_t>(grp * 32) << 16) +
                            static_cast<uint32_t>(acc * Cfg::ACC_COLS);
-    float* mypart = g.partial + (static_cast<size_t>(u) * g.maxc + slot) * g.bn * kBM;
-    // Split-K: the unit's contributors are CTAs first..last (slots 0..nc-1).
-    // Slot 0 -- for which this unit is the last segment of its range, so it
+    float* mypart = g.partial + (static_cast<size_t>(mt) * g.maxc + slot) * g.bn * kBM;
+    // Split-K: the tile's contributors are ranges first..last (slots 0..nc-1).
+    // Slot 0 -- for which this tile is the last segment of its range, so it
     // finishes with the phase -- owns the reduction: the others store their
     // partial sums and release a count; the owner waits for nc - 1, then adds
     // the partials to its own accumulator in slot order.
@@ -479,19 +531,22 @@ __device__ bool tc_epilogue(const TcPipe& P, int& acc, uint32_t& accph, const Ge
         float v[kEpiCols];
         tmem_ld_sum_cfg<Cfg>(taddr, ch, g.bn, v);
         if (nc == 1) {
-          epi_apply<KIND, __nv_bfloat16>(e, mt, tbase + ch * kEpiCols, v, r, es, &pre);
+          epi_apply<KIND, __nv_bfloat16>(e, mt, ch * kEpiCols, v, r, es, use_pre);
         } else {
+          if constexpr (PAIR) {
+            part_st16(mypart, ch, r, v);
+          } else {
 #pragma unroll
-          for (int j = 0; j < kEpiCols; ++j) mypart[(ch * kEpiCols + j) * kBM + r] = v[j];
+            for (int j = 0; j < kEpiCols; ++j) mypart[(ch * kEpiCols + j) * kBM + r] = v[j];
+          }
         }
       }
       if (nc == 1) epi_publish(e, mt, r);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&P.tempty[acc]);
+      release();
       if (nc > 1) {
+        if constexpr (PAIR) asm volatile("fence.proxy.async.global;" ::: "memory");  // (read by bulk copies)
         joint();  // every thread's partial stores precede the release
-        if (gi == 0 && r == 0) red_release_gpu(&g.tickets[u], 1);
+        if (gi == 0 && r == 0) red_release_gpu(&g.tickets[mt], 1);
         if (dbg) e.dbg[e.dbg_stride + cta] = globaltimer_ns();
       } else if (KIND == EPI_ARGMAX) {
         if constexpr (NG > 1) joint();  // both groups' partial maxima are written
@@ -501,63 +556,110 @@ __device__ bool tc_epilogue(const TcPipe& P, int& acc, uint32_t& accph, const Ge
       bool got;
       if constexpr (NG > 1) {
         // one wait for both groups, so that they agree on its outcome
-        if (gi == 0 && r == 0) *P.jflag = count_wait(&g.tickets[u], nc - 1, P.abort) ? 1 : 0;
+        if (gi == 0 && r == 0) *P.jflag = count_wait(&g.tickets[mt], nc - 1, P.abort) ? 1 : 0;
         joint();
         got = *P.jflag != 0;
       } else {
-        if (r == 0) es.ok = count_wait(&g.tickets[u], nc - 1, P.abort) ? 1 : 0;
+        if (r == 0) es.ok = count_wait(&g.tickets[mt], nc - 1, P.abort) ? 1 : 0;
         epi_sync();
         got = es.ok != 0;
         epi_sync();
       }
       if (!got) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&P.tempty[acc]);
+        release();
         return false;
       }
       if (dbg) e.dbg[e.dbg_stride + cta] = globaltimer_ns();
-      for (int ch = gi; ch < nchunk; ch += NG) {
-        float v[kEpiCols];
-        tmem_ld_sum_cfg<Cfg>(taddr, ch, g.bn, v);
-        // slots 1..nc-1: a group of up to red_slots partial blocks
-        // (kEpiCols x kBM contiguous floats each) is copied to shared memory
-        // by all 128 threads at once (cp.async at L2, no registers held),
-        // then each thread adds its row
-        for (int s0 = 1; s0 < nc; s0 += P.red_slots) {
-          const int ns = min(P.red_slots, nc - s0);
-          for (int q = 0; q < ns; ++q) {
-            const float* src = g.partial + (static_cast<size_t>(u) * g.maxc + s0 + q) * g.bn * kBM +
-                               static_cast<size_t>(ch) * kEpiCols * kBM;
-            float* dst = P.red + q * (kEpiCols * kBM);
+      if constexpr (PAIR) {
+        // This is the CTA's last segment, so its ring is idle: the partials
+        // of slots 1..nc-1 come through it by bulk copies (per-thread loads
+        // reached 30 GB/s), a round of four chunks of one slot per buffer, three
+        // rounds in flight per group; the totals go back to tensor memory
+        // (the hi columns).
+        const int mine = (nchunk - gi + NG - 1) / NG;  // this group's chunks
+        const int per = nc - 1, rounds = (mine + 3) / 4 * per;
+        uint8_t* buf = P.ring_free + gi * (kPartRounds * 4 * kPartChunkBytes);
+        uint64_t* bar = P.part_bar + gi * kPartRounds;
+        auto load_round = [&](int k) {
+          const int cb = (k / per) * 4, s0 = 1 + k % per, n = min(4, mine - cb);
+          const float* src = g.partial + (static_cast<size_t>(mt) * g.maxc + s0) * g.bn * kBM;
+          uint64_t* b = bar + k % kPartRounds;
+          mbar_arrive_expect_tx(b, n * kPartChunkBytes);
+          for (int i = 0; i < n; ++i)
+            bulk_load(buf + ((k % kPartRounds) * 4 + i) * kPartChunkBytes,
+                      src + static_cast<size_t>(gi + (cb + i) * NG) * (kEpiCols * kBM), kPartChunkBytes, b);
+        };
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        if (r == 0)
+          for (int k = 0; k < min(rounds, kPartRounds); ++k) load_round(k);
+        bool got_all = true;
+        for (int k = 0, cb = 0; cb < mine; cb += 4) {
+          float v[4][kEpiCols];
 #pragma unroll
-            for (int i = 0; i < kEpiCols * kBM / (4 * 128); ++i)
-              cp_async16(dst + 4 * (i * 128 + r), src + 4 * (i * 128 + r));
-          }
-          cp_async_commit();
-          // the chunk's own epilogue inputs travel in the same round trip
-          if (ch > gi && s0 == 1)
-            epi_prefetch<KIND, __nv_bfloat16>(e, mt, tbase + ch * kEpiCols, r, es, pre);
-          cp_async_wait_all();
-          epi_sync();
-          for (int q = 0; q < ns; ++q) {
-            const float* blk = P.red + q * (kEpiCols * kBM);
+          for (int i = 0; i < 4; ++i)
+            if (cb + i < mine) tmem_ld_sum_cfg<Cfg>(taddr, gi + (cb + i) * NG, g.bn, v[i]);
+          for (int s0 = 1; s0 < nc; ++s0, ++k) {
+            // (bounded, and not cut short by another role's abort: the copy must land)
+            got_all &= mbar_wait(bar + k % kPartRounds, (k / kPartRounds) & 1, nullptr);
+            const uint8_t* b = buf + (k % kPartRounds) * 4 * kPartChunkBytes;
 #pragma unroll
-            for (int j = 0; j < kEpiCols; ++j) v[j] += blk[j * kBM + r];
+            for (int i = 0; i < 4; ++i)
+              if (cb + i < mine) part_add16(v[i], b + i * kPartChunkBytes, r);
+            epi_sync();  // the buffer has been read
+            if (r == 0 && k + kPartRounds < rounds) load_round(k + kPartRounds);
           }
-          epi_sync();
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (cb + i < mine) tmem_st16(taddr + (gi + (cb + i) * NG) * kEpiCols, v[i]);
         }
-        if (dbg && ch == 0) e.dbg[4 * e.dbg_stride + cta] = globaltimer_ns();
-        epi_apply<KIND, __nv_bfloat16>(e, mt, tbase + ch * kEpiCols, v, r, es, &pre);
+        tmem_st_wait();
+        if (!got_all) *P.abort = 1;  // (the sums are incomplete: the launch reports a timeout)
+        for (int ch = gi; ch < nchunk; ch += NG) {
+          float v[kEpiCols];
+          tmem_ld16(taddr + ch * kEpiCols, v);
+          epi_apply<KIND, __nv_bfloat16>(e, mt, ch * kEpiCols, v, r, es, use_pre);
+        }
+      } else {
+        for (int ch = gi; ch < nchunk; ch += NG) {
+          float v[kEpiCols];
+          tmem_ld_sum_cfg<Cfg>(taddr, ch, g.bn, v);
+          // slots 1..nc-1: a group of up to red_slots partial blocks
+          // (kEpiCols x kBM contiguous floats each) is copied to shared memory
+          // by all 128 threads at once (cp.async at L2, no registers held),
+          // then each thread adds its row
+          for (int s0 = 1; s0 < nc; s0 += P.red_slots) {
+            const int ns = min(P.red_slots, nc - s0);
+            for (int q = 0; q < ns; ++q) {
+              const float* src = g.partial + (static_cast<size_t>(mt) * g.maxc + s0 + q) * g.bn * kBM +
+                                 static_cast<size_t>(ch) * kEpiCols * kBM;
+              float* dst = P.red + q * (kEpiCols * kBM);
+#pragma unroll
+              for (int i = 0; i < kEpiCols * kBM / (4 * 128); ++i)
+                cp_async16(dst + 4 * (i * 128 + r), src + 4 * (i * 128 + r));
+            }
+            cp_async_commit();
+            // the chunk's own epilogue inputs travel in the same round trip
+            if (ch > gi && s0 == 1)
+              epi_prefetch<KIND, __nv_bfloat16>(e, mt, ch * kEpiCols, r, es, pre);
+            cp_async_wait_all();
+            epi_sync();
+            for (int q = 0; q < ns; ++q) {
+              const float* blk = P.red + q * (kEpiCols * kBM);
+#pragma unroll
+              for (int j = 0; j < kEpiCols; ++j) v[j] += blk[j * kBM + r];
+            }
+            epi_sync();
+          }
+          if (dbg && ch == 0) e.dbg[4 * e.dbg_stride + cta] = globaltimer_ns();
+          epi_apply<KIND, __nv_bfloat16>(e, mt, ch * kEpiCols, v, r, es, use_pre);
+        }
       }
       // (the count is reset before the tile is published: a later phase that
       // the flag opens may count on the same ticket)
       if constexpr (NG > 1) joint();  // both groups are past the wait and done
-      if (gi == 0 && r == 0) g.tickets[u] = 0;
+      if (gi == 0 && r == 0) g.tickets[mt] = 0;
       epi_publish(e, mt, r);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&P.tempty[acc]);
+      release();
       if (KIND == EPI_ARGMAX && gi == 0) epi_argmax_finish(e, r, es);
     }
     if (dbg) e.dbg[2 * e.dbg_stride + cta] = globaltimer_ns();

@@ -73,6 +73,7 @@ struct WideSmem {
 };
 
 constexpr size_t wide_smem_bytes() { return 1024 + kWStages * kWStage + sizeof(WideSmem); }
+static_assert(kWideTokens == 8 * kEpiCols, "partial layout");
 static_assert(wide_smem_bytes() <= 227 * 1024, "wide GEMM shared memory");
 
 // (max, argmax, second max) of 16 columns over a warp's 32 rows; column c ends
@@ -275,6 +276,20 @@ __device__ __forceinline__ void wide_apply(const EpiArgs& e, const GemmArgs& g, 
         dst[2] = b2;
       }
     }
+  }
+}
+
+__device__ __forceinline__ void part_add16_global(const float* part, int ch, int r, float (&v)[kEpiCols]) {
+  const float4* p = reinterpret_cast<const float4*>(part) + static_cast<size_t>(ch) * 4 * kBM + r;
+  float4 t[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) t[q] = __ldcg(p + q * kBM);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    v[4 * q] += t[q].x;
+    v[4 * q + 1] += t[q].y;
+    v[4 * q + 2] += t[q].z;
+    v[4 * q + 3] += t[q].w;
   }
 }
 
@@ -496,10 +511,16 @@ __global__ void __launch_bounds__(kWThreads, 1)
       const bool owner = cluster == first;
       if (owner && KIND != EPI_RESID && KIND != EPI_ACC) {
         // the unit's RMSNorm scales, positions and sequences, while its MMAs run
-        for (int tb = 0; tb < g.bn; tb += 32) {
-          const int tl = tb + (et >> 3), t = t0 + tl;
-          const float ss = epi_ssq_column(e, t, et & 7, tl < g.bn && t < e.T);
-          if ((et & 7) == 0 && tl < g.bn) s.rs[tl] = t < e.T ? rsqrtf(ss * e.inv_d + e.eps) : 0.f;
+        const int tq = (et >> 3) * 4, part = et & 7;
+        if ((et & ~31) / 2 < g.bn) {  // (a warp's 4 column quads; bn is a multiple of 16)
+          const bool in = t0 + tq < e.T;
+          float ss[4];
+          epi_ssq_quad(e, in ? t0 + tq : 0, part, ss);
+          if (part < 4)
+            s.rs[tq + part] = t0 + tq + part < e.T
+                                  ? rsqrtf((part == 0 ? ss[0] : part == 1 ? ss[1] : part == 2 ? ss[2] : ss[3]) * e.inv_d +
+                                           e.eps)
+                                  : 0.f;
         }
         if (KIND == EPI_QKV && et < g.bn) {
           s.pos[et] = t0 + et < e.T ? e.pos[t0 + et] : 0;
@@ -524,16 +545,12 @@ __global__ void __launch_bounds__(kWThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_remote(tempty_leader);  // the next unit's MMAs may start
       if (!owner) {
-        float* part = g.partial + (static_cast<size_t>(cluster) * kCl + crank) * kWidePartFloats + lr;
+        float* part = g.partial + (static_cast<size_t>(cluster) * kCl + crank) * kWidePartFloats;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const int tl = (grp + 2 * q) * kEpiCols;
-          if (tl < g.bn) {
-#pragma unroll
-            for (int j = 0; j < kEpiCols; ++j) {
-              __stcg(part + (tl + j) * kBM, v0[q][j]);
-              __stcg(part + (kWideTokens + tl + j) * kBM, v1[q][j]);
-            }
+          if ((grp + 2 * q) * kEpiCols < g.bn) {
+            part_st16(part, grp + 2 * q, lr, v0[q]);
+            part_st16(part, 8 + grp + 2 * q, lr, v1[q]);
           }
         }
         joint();  // every thread's stores precede the release
@@ -545,16 +562,12 @@ __global__ void __launch_bounds__(kWThreads, 1)
         joint();
         if (!s.ok[1]) break;
         for (int o = first + 1; o <= last; ++o) {
-          const float* part = g.partial + (static_cast<size_t>(o) * kCl + crank) * kWidePartFloats + lr;
+          const float* part = g.partial + (static_cast<size_t>(o) * kCl + crank) * kWidePartFloats;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const int tl = (grp + 2 * q) * kEpiCols;
-            if (tl < g.bn) {
-#pragma unroll
-              for (int j = 0; j < kEpiCols; ++j) {
-                v0[q][j] += __ldcg(part + (tl + j) * kBM);
-                v1[q][j] += __ldcg(part + (kWideTokens + tl + j) * kBM);
-              }
+            if ((grp + 2 * q) * kEpiCols < g.bn) {
+              part_add16_global(part, grp + 2 * q, lr, v0[q]);
+              part_add16_global(part, 8 + grp + 2 * q, lr, v1[q]);
             }
           }
         }

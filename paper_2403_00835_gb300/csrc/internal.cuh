@@ -81,11 +81,13 @@ struct EpiArgs {
 
 // Work decomposition of one weight-streaming GEMM launch.
 //   D[m][t] = sum_k W[m][k] X[t][k]  (m: weight rows, t: tokens)
-// The chunk space (unit, k-chunk) is split into contiguous ranges of `cpc`
-// chunks, one per CTA; a unit is one 128-row tile x one N-tile of tokens.
+// Up to 256 tokens: the (group of 128-row tiles, k-chunk) space is split into
+// contiguous ranges of `cpc` chunks, one per CTA of each tile residue (see
+// cta_range); every token is in the one N tile.
 struct GemmArgs {
   int M, K, T;
   int mtiles, ntiles, kchunks, cpc, bn, maxc;
+  int gshift;           // log2 of the tiles per group
   int rows_q, rows_qk;  // QKV: first rows of the K and V sections (weight-map select)
   int lo_rows;          // row offset of the activations' lo plane in the B map
   int l2_ahead;         // weight tiles per CTA prefetched into L2 before the PDL wait
@@ -292,10 +294,18 @@ inline int round_up(int a, int b) { return ceil_div(a, b) * b; }
 struct Part {
   int mtiles, ntiles, kchunks, cpc, bn, bn_max, maxc, grid;
 };
-Part plan_gemm(int mtiles, int K, int T, int sms);
+Part plan_gemm(int mtiles, int K, int T, int sms);   // a stand-alone GEMM: single-tile groups
+constexpr int kGroupShift = 2;
+Part plan_group(int mtiles, int K, int T, int sms);  // the engine's launches of up to 256 tokens
 // bf16 [outer][inner] tensor map: 64-column x box_outer-row tiles, 128-byte swizzle.
 bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint32_t box_outer);
 
+// up to 256 tokens, plan_group's split (gemm_pair.cu); the activation map's box has
+// pair_box_rows(bn) rows
+cudaError_t launch_gemm_pair(int kind, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int grid,
+                             cudaStream_t s, bool pdl);
+cudaError_t gemm_pair_set_attributes();
+inline int pair_box_rows(int bn) { return bn <= 128 ? bn : bn / 2; }
 
 // Wide launches (T > 256, gemm_wide.cu): units of 512 weight rows (gate/up:
 // 256 features) x bn tokens per CTA pair, the (unit, K chunk) space in ranges
@@ -348,8 +358,6 @@ cudaError_t launch_gather_rows(const void* xg_src, const float* ssq_src, void* x
                                float* ssq_dst, const int* rows, int B, int d, int ldt_src,
                                int ldt_dst, size_t plane_src, size_t plane_dst, int act_bf16,
                                cudaStream_t s);
-int gemm_tc_stages(int bn_max);
-size_t gemm_tc_smem_bytes(int bn_max);
 cudaError_t gemm_tc_set_attributes();
 cudaError_t gemm_tc_set_attributes_acc(int bn_max);  // EPI_ACC, one column count
 cudaError_t attention_set_attributes();

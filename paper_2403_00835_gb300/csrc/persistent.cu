@@ -192,9 +192,9 @@ constexpr int kMaxWeightPairs = 2;
 template <int KIND, class PC>
 __device__ __forceinline__ void pk_load_a_chunk(uint8_t* dst, uint64_t* bar, const GemmArgs& g,
                                                 const CUtensorMap* mA0, const CUtensorMap* mA1,
-                                                const CUtensorMap* mA2, int c, uint64_t pol) {
+                                                const CUtensorMap* mA2, int c, int cta, uint64_t pol) {
   const int u = c / g.kchunks, k = c - u * g.kchunks;
-  const int mt = u / g.ntiles;
+  const int mt = tile_of(g, u, cta);
   if (KIND == EPI_GATEUP) {
     tma_load_2d(dst, mA0, bar, k * kBK, mt * 64, pol);
     tma_load_2d(dst + PC::A_CHUNK / 2, mA1, bar, k * kBK, mt * 64, pol);
@@ -214,9 +214,9 @@ __device__ __forceinline__ void pk_load_a_chunk(uint8_t* dst, uint64_t* bar, con
 template <int KIND>
 __device__ __forceinline__ void pk_prefetch_chunk(const GemmArgs& g, const CUtensorMap* mA0,
                                                   const CUtensorMap* mA1, const CUtensorMap* mA2,
-                                                  int c) {
+                                                  int c, int cta) {
   const int u = c / g.kchunks, k = c - u * g.kchunks;
-  const int mt = u / g.ntiles;
+  const int mt = tile_of(g, u, cta);
   if (KIND == EPI_GATEUP) {
     tma_prefetch_l2_2d(mA0, k * kBK, mt * 64);
     tma_prefetch_l2_2d(mA1, k * kBK, mt * 64);
@@ -236,7 +236,7 @@ __device__ __forceinline__ void pk_prefetch_chunk(const GemmArgs& g, const CUten
 template <int KIND, class PC>
 __device__ bool pk_produce_a(const PkPipe& P, int& ia, const GemmArgs& g, const CUtensorMap* mA0,
                              const CUtensorMap* mA1, const CUtensorMap* mA2, int c0, int c1,
-                             int l2_ahead) {
+                             int cta, int l2_ahead) {
   constexpr int S = PC::SA;
   const uint64_t pol_w = l2_policy_evict_first();
   int pf = c0;  // next chunk of this phase to prefetch into L2
@@ -247,7 +247,7 @@ __device__ bool pk_produce_a(const PkPipe& P, int& ia, const GemmArgs& g, const 
       // can): fetch the phase's next tiles into L2 meanwhile
       if (pf < c + kPairChunks) pf = c + kPairChunks;
       for (; pf < c1 && pf < c + kPairChunks * (1 + l2_ahead); ++pf)
-        pk_prefetch_chunk<KIND>(g, mA0, mA1, mA2, pf);
+        pk_prefetch_chunk<KIND>(g, mA0, mA1, mA2, pf, cta);
     }
     if (!mbar_wait(&P.aempty[st], ((ia / S) & 1) ^ 1, P.abort)) return false;
     if (S > kMaxWeightPairs && ia >= kMaxWeightPairs) {  // at most kMaxWeightPairs in flight
@@ -256,8 +256,8 @@ __device__ bool pk_produce_a(const PkPipe& P, int& ia, const GemmArgs& g, const 
     }
     mbar_arrive_expect_tx(&P.afull[st], PC::A_BYTES);
     uint8_t* dst = P.sA + st * PC::A_BYTES;
-    pk_load_a_chunk<KIND, PC>(dst, &P.afull[st], g, mA0, mA1, mA2, c, pol_w);
-    pk_load_a_chunk<KIND, PC>(dst + PC::A_CHUNK, &P.afull[st], g, mA0, mA1, mA2, c + 1, pol_w);
+    pk_load_a_chunk<KIND, PC>(dst, &P.afull[st], g, mA0, mA1, mA2, c, cta, pol_w);
+    pk_load_a_chunk<KIND, PC>(dst + PC::A_CHUNK, &P.afull[st], g, mA0, mA1, mA2, c + 1, cta, pol_w);
   }
   return true;
 }
@@ -337,19 +337,15 @@ __device__ bool pk_produce_b(const PkPipe& P, int& ib, const GemmArgs& g, const 
   }
   const uint64_t pol_x = l2_policy_evict_last();
   const uint32_t b_bytes = 2u * static_cast<uint32_t>(g.bn) * kBK * 2;
-  const bool tile_mode = g.ntiles > 1;
   for (int c = c0; c < c1; c += kPairChunks, ++ib) {
     const int st = ib % S;
     if (!mbar_wait(&P.bempty[st], ((ib / S) & 1) ^ 1, P.abort)) return false;
     mbar_arrive_expect_tx(&P.bfull[st], kPairChunks * b_bytes);
     for (int h = 0; h < kPairChunks; ++h) {
-      const int cc = c + h;
-      const int u = cc / g.kchunks, k = cc - u * g.kchunks;
-      const int nt = u % g.ntiles;
-      const int row0 = tile_mode ? nt * PC::BN : 0;
+      const int k = (c + h) % g.kchunks;
       uint8_t* dst = P.sB + st * PC::B_BYTES + h * PC::B_REGION;
-      tma_load_2d(dst, mB, &P.bfull[st], k * kBK, row0, pol_x);
-      tma_load_2d(dst + g.bn * kBK * 2, mB, &P.bfull[st], k * kBK, g.lo_rows + row0, pol_x);
+      tma_load_2d(dst, mB, &P.bfull[st], k * kBK, 0, pol_x);
+      tma_load_2d(dst + g.bn * kBK * 2, mB, &P.bfull[st], k * kBK, g.lo_rows, pol_x);
     }
   }
   return true;
@@ -505,9 +501,9 @@ __device__ bool produce_a_phase(const PkPipe& P, int& ia, const PhaseDesc& ph,
   int c0, c1;
   cta_range(g, cta, c0, c1);
   switch (ph.epi) {
-    case EPI_QKV: return pk_produce_a<EPI_QKV, PC>(P, ia, g, m0, m1, m2, c0, c1, l2_ahead);
-    case EPI_GATEUP: return pk_produce_a<EPI_GATEUP, PC>(P, ia, g, m0, m1, m2, c0, c1, l2_ahead);
-    default: return pk_produce_a<EPI_RESID, PC>(P, ia, g, m0, m1, m2, c0, c1, l2_ahead);
+    case EPI_QKV: return pk_produce_a<EPI_QKV, PC>(P, ia, g, m0, m1, m2, c0, c1, cta, l2_ahead);
+    case EPI_GATEUP: return pk_produce_a<EPI_GATEUP, PC>(P, ia, g, m0, m1, m2, c0, c1, cta, l2_ahead);
+    default: return pk_produce_a<EPI_RESID, PC>(P, ia, g, m0, m1, m2, c0, c1, cta, l2_ahead);
   }
 }
 
