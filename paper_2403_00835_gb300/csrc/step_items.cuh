@@ -30,10 +30,8 @@ __device__ __forceinline__ int draw_guess(const AcceptArgs& a, int b, int step, 
   return static_cast<int>((r * static_cast<uint64_t>(a.V)) >> 32);
 }
 
-template <typename Act, class Sync>
-__device__ void embed_unit(const EmbedArgs& a, int t, int grp, int i, float* red, Sync sync) {
-  const int m = grp * 128 + i;
-  int tok, pos, b;
+// Token, position and sequence of row t.
+__device__ __forceinline__ void embed_row(const EmbedArgs& a, int t, int& tok, int& pos, int& b) {
   if (a.block != nullptr) {
     b = t / a.n;
     const int k = t - b * a.n;
@@ -44,6 +42,30 @@ __device__ void embed_unit(const EmbedArgs& a, int t, int grp, int i, float* red
     pos = a.pos_in[t];
     b = a.bidx_in[t];
   }
+}
+
+// Row t's position and sequence index; with row 0, the sequences' row ranges
+// (threads i = 0 .. n - 1 of the row's first group call).
+__device__ __forceinline__ void embed_meta(const EmbedArgs& a, int t, int pos, int b, int i, int n) {
+  if (i == 0) {
+    if (pos < 0 || pos >= a.max_seq) atomicOr(a.err, DERR_CAPACITY);
+    a.pos[t] = pos;
+    a.bidx[t] = b;
+  }
+  if (a.block != nullptr && t == 0) {
+    for (int bb = i; bb < a.B; bb += n) {
+      a.seq_start[bb] = a.L[bb];
+      a.seq_row0[bb] = bb * a.n;
+      a.seq_nrows[bb] = a.n;
+    }
+  }
+}
+
+template <typename Act, class Sync>
+__device__ void embed_unit(const EmbedArgs& a, int t, int grp, int i, float* red, Sync sync) {
+  const int m = grp * 128 + i;
+  int tok, pos, b;
+  embed_row(a, t, tok, pos, b);
   if (tok < 0 || tok >= a.V) {
     if (i == 0 && grp == 0) atomicOr(a.err, DERR_TOKEN);
     tok = 0;
@@ -56,18 +78,7 @@ __device__ void embed_unit(const EmbedArgs& a, int t, int grp, int i, float* red
   if ((i & 31) == 0) red[i >> 5] = s;
   sync();
   if (i == 0) a.ssq[static_cast<size_t>(grp) * a.ldt + t] = ((red[0] + red[1]) + red[2]) + red[3];
-  if (grp == 0 && i == 0) {
-    if (pos < 0 || pos >= a.max_seq) atomicOr(a.err, DERR_CAPACITY);
-    a.pos[t] = pos;
-    a.bidx[t] = b;
-  }
-  if (a.block != nullptr && t == 0 && grp == 0) {
-    for (int bb = i; bb < a.B; bb += 128) {
-      a.seq_start[bb] = a.L[bb];
-      a.seq_row0[bb] = bb * a.n;
-      a.seq_nrows[bb] = a.n;
-    }
-  }
+  if (grp == 0) embed_meta(a, t, pos, b, i, 128);
   sync();  // red[] is reused by the next unit
 }
 
