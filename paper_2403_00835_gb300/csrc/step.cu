@@ -107,20 +107,25 @@ __global__ void set_head_kernel(int* block, const int* head, int B, int n, int V
   }
 }
 
-template <typename Act>
-__global__ void gather_rows_kernel(const Act* xg_src, const float* ssq_src, Act* xg_dst,
-                                   float* ssq_dst, const int* rows, int d, int ldt_src,
-                                   int ldt_dst, size_t plane_src, size_t plane_dst) {
-  const int b = blockIdx.x;
-  const int row = rows[b];
-  for (int m = threadIdx.x; m < d; m += blockDim.x) {
-    xg_dst[static_cast<size_t>(b) * d + m] = xg_src[static_cast<size_t>(row) * d + m];
-    if (plane_dst)
-      xg_dst[plane_dst + static_cast<size_t>(b) * d + m] =
-          xg_src[plane_src + static_cast<size_t>(row) * d + m];
+// Row `rows[b]` of the norm input (row_bytes per plane, 16-byte pieces; the lo
+// plane, if any, plane bytes further) and of its statistics.  Every piece is
+// one independent load, so a row costs one round trip (element by element it
+// took 17 us).
+__global__ void __launch_bounds__(256) gather_rows_kernel(const char* src, const float* ssq_src, char* dst,
+                                                          float* ssq_dst, const int* rows, int row_bytes, int d,
+                                                          int ldt_src, int ldt_dst, size_t plane_src,
+                                                          size_t plane_dst) {
+  const int b = blockIdx.x, row = rows[b];
+  const int per = row_bytes / 16, n = plane_dst ? 2 * per : per;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 256) {
+    const int pl = i >= per ? 1 : 0;
+    const size_t o = static_cast<size_t>(i - pl * per) * 16;
+    *reinterpret_cast<uint4*>(dst + pl * plane_dst + static_cast<size_t>(b) * row_bytes + o) =
+        __ldcg(reinterpret_cast<const uint4*>(src + pl * plane_src + static_cast<size_t>(row) * row_bytes + o));
   }
-  for (int i = threadIdx.x; i < d / 128; i += blockDim.x)
-    ssq_dst[static_cast<size_t>(i) * ldt_dst + b] = ssq_src[static_cast<size_t>(i) * ldt_src + row];
+  for (int i = threadIdx.x; i < d / 128; i += 256)
+    ssq_dst[static_cast<size_t>(i) * ldt_dst + b] = __ldcg(ssq_src + static_cast<size_t>(i) * ldt_src + row);
 }
 
 // ---- launchers ----------------------------------------------------------------------
@@ -167,14 +172,11 @@ cudaError_t launch_gather_rows(const void* xg_src, const float* ssq_src, void* x
                                float* ssq_dst, const int* rows, int B, int d, int ldt_src,
                                int ldt_dst, size_t plane_src, size_t plane_dst, int act_bf16,
                                cudaStream_t s) {
-  if (act_bf16)
-    gather_rows_kernel<__nv_bfloat16><<<B, 256, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(xg_src), ssq_src, static_cast<__nv_bfloat16*>(xg_dst),
-        ssq_dst, rows, d, ldt_src, ldt_dst, plane_src, plane_dst);
-  else
-    gather_rows_kernel<float><<<B, 256, 0, s>>>(static_cast<const float*>(xg_src), ssq_src,
-                                                static_cast<float*>(xg_dst), ssq_dst, rows, d,
-                                                ldt_src, ldt_dst, 0, 0);
+  // (d is a multiple of 128, so rows and planes are whole 16-byte pieces)
+  const size_t es = act_bf16 ? 2 : 4;
+  gather_rows_kernel<<<B, 256, 0, s>>>(static_cast<const char*>(xg_src), ssq_src, static_cast<char*>(xg_dst), ssq_dst,
+                                       rows, static_cast<int>(d * es), d, ldt_src, ldt_dst,
+                                       act_bf16 ? plane_src * es : 0, act_bf16 ? plane_dst * es : 0);
   return cudaGetLastError();
 }
 
