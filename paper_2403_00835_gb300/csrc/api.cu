@@ -60,11 +60,10 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, 
 // Split of one stand-alone GEMM over the SMs.  T <= 256: one N-tile holding every
 // token and the (tile, k-chunk) space cut into equal contiguous ranges; the
 // cut depends on the weight shape and the SM count only.  T > 256: whole
-// 128 x 256 tiles per CTA, no split.  Chunks per tile and per CTA are even,
-// so that every range and every tile starts on a pair of chunks: the
-// persistent kernel moves weights in pairs (32 KB per pipeline stage), in the
-// same order as the per-chunk kernels, which keeps the two paths bit-identical.
-// (A K that is not a multiple of 128 gets one chunk past its end, which TMA
+// 128 x 256 tiles per CTA, no split (launches of that size run plan_wide's
+// split; this one bounds what the allocation-free entry point accepts).  Chunks
+// per tile and per CTA are even.  (A K that is not a multiple of 128 gets one
+// chunk past its end, which TMA
 // fills with zeros.)
 Part plan_gemm(int mtiles, int K, int T, int sms) {
   Part p{};

@@ -1,7 +1,7 @@
 // The three warp roles of the weight-streaming GEMM, as device functions that
-// carry their pipeline state across calls.  A standalone GEMM kernel runs one
-// phase; the persistent per-iteration kernel runs many phases back to back on
-// the same shared-memory ring and TMEM accumulators.
+// carry their pipeline state across calls.  The stand-alone GEMM kernel runs one
+// phase; the persistent per-iteration kernel (its own producer and MMA roles)
+// runs many phases' epilogues back to back, and the CTA-pair kernel one.
 //
 //   producer (one thread): TMA of weight tiles (A, evict-first) and the
 //     activation tile's hi/lo planes (B, evict-last) into the stage ring.
@@ -9,8 +9,8 @@
 //     the phase's dependency (previous kernel / grid barrier) is satisfied;
 //     activation tiles only after.
 //   MMA issuer (one thread): tcgen05.mma M=128 into a TMEM accumulator pair.
-//   epilogue (warps 2..5, 128 threads): tcgen05.ld, split-K partials with a
-//     last-arriver fixed-order reduction, fused epilogue (epilogue.cuh).
+//   epilogue (warps 2..5, 128 threads): tcgen05.ld, split-K partials reduced in
+//     a fixed order by the tile's first contributor, fused epilogue (epilogue.cuh).
 #pragma once
 #include "epilogue.cuh"
 
