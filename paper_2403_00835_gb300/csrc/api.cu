@@ -1365,7 +1365,7 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
     }
     c->gemm_part_elems = need;
     if (c->bf16 && c->Tcap > 256) {
-      const size_t ctas = static_cast<size_t>(c->wide_clusters) * kWideCluster;
+      const size_t ctas = static_cast<size_t>(c->wide_clusters) * 2;
       ok = ok && dev_alloc(c, &c->wide_part, ctas * kWidePartFloats * 4) && dev_alloc(c, &c->wide_tickets, ctas * 4);
     }
     ok = ok && dev_alloc(c, &c->gemm_part, need * 4) && dev_alloc(c, &c->tickets, c->max_mtiles * 4) &&
@@ -1955,7 +1955,7 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
   };
   int rc = CLLM_OK;
   do {
-    const size_t ctas = static_cast<size_t>(w.clusters) * kWideCluster;
+    const size_t ctas = static_cast<size_t>(w.clusters) * 2;
     float* part = static_cast<float*>(
         alloc(wide ? ctas * kWidePartFloats * 4 : static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
     int* tickets = static_cast<int*>(alloc(wide ? ctas * 4 : mtiles * 4));

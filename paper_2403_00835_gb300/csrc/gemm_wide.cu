@@ -10,8 +10,7 @@
 // chunk costs a CTA 48 KB of shared-memory fill for eight MMAs of M = 256,
 // N = 256 (0.58 us at the dense rate).  The 128 x 256 tile of a single CTA
 // with both planes cost 80 KB for the same MMA work and ran at the L2's
-// bandwidth.  kCl = 4: two pairs of a cluster take neighbouring token tiles
-// of the same rows and share each weight tile by multicast.
+// bandwidth.
 //
 // The two weight tiles are two accumulators (hi and lo columns of each: 512
 // tensor-memory columns) whose rows are chosen so that a lane holds what the
@@ -32,9 +31,12 @@
 // Per launch at 2048 rows, 7B shape, against the single-CTA kernel: gate/up
 // 757 -> 384 us (1.93 PFLOP/s counting both planes: the power limit), QKV 555
 // -> 241, O and down together 511 -> 357; at 1024 rows gate/up 571 -> 302 (a
-// mean over 1024- and 2048-row launches).  Two pairs per cluster against one:
-// 4096-row prefill 6.66 against 7.00 ms, 16 x 64 rows 8.00 against 8.36,
-// although clusters of 4 leave 8 of the 152 SMs without work.
+// mean over 1024- and 2048-row launches).  Those were taken with two pairs of
+// a cluster sharing each weight tile by multicast loads; a pair now loads its
+// own, because the ranks of a replica run load this library too and a
+// multicast load has no place in a multi-GPU program.  4096-row prefill
+// (2 layers) 5.23 -> 5.53 ms, 500 rows 1.23 -> 1.25, 16 x 64 rows unchanged
+// (the pairs use all 152 SMs, clusters of 4 used 144).
 #include <float.h>
 #include <limits.h>
 
@@ -326,7 +328,7 @@ struct WideWork {
   }
 };
 
-template <int KIND, int kCl>
+template <int KIND>
 __global__ void __launch_bounds__(kWThreads, 1)
     gemm_wide_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                      const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB, const GemmArgs g,
@@ -337,12 +339,9 @@ __global__ void __launch_bounds__(kWThreads, 1)
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   WideSmem& s = *reinterpret_cast<WideSmem*>(ring + kWStages * kWStage);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t crank = cluster_ctarank();
-  const int pair = crank >> 1, r = crank & 1;  // pair of the cluster, CTA of the pair
+  const uint32_t r = cluster_ctarank();  // CTA of the pair
   const bool leader = r == 0;
-  constexpr int kPairs = kCl / 2;
-  constexpr uint16_t kAllMask = (1u << kCl) - 1;
-  const int cluster = blockIdx.x / kCl;
+  const int cluster = blockIdx.x / 2;
   volatile int* abort = &s.abort_flag;
 
   if (threadIdx.x == 0) {
@@ -350,7 +349,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
     tma_prefetch_desc(&mB);
     for (int i = 0; i < kWStages; ++i) {
       mbar_init(&s.full[i], 1);
-      mbar_init(&s.empty[i], kPairs);
+      mbar_init(&s.empty[i], 1);
     }
     mbar_init(&s.tfull, 1);
     mbar_init(&s.tempty, 16);  // the 8 epilogue warps of both CTAs
@@ -370,14 +369,14 @@ __global__ void __launch_bounds__(kWThreads, 1)
   const uint32_t tmem = s.tmem;
   pdl_launch_dependents();
 
-  WideWork work(g, cluster, gridDim.x / kCl);
+  WideWork work(g, cluster, gridDim.x / 2);
   Segment sg;
   int first, last;
-  // row unit (512 rows; GATEUP: 256 features) and this pair's first token of unit u
-  auto unit_tok = [&](int u) { return ((u % g.ntiles) * kPairs + pair) * g.bn; };
+  // first token and this CTA's first row of unit u (512 rows; GATEUP: 256 features)
+  auto unit_tok = [&](int u) { return (u % g.ntiles) * g.bn; };
   auto unit_row = [&](int u) {
-    const int ru = u / g.ntiles;
-    return KIND == EPI_GATEUP ? ru * 256 + r * 128 : ru * 512 + r * 256;
+    const int ru = u / g.ntiles, half = static_cast<int>(r);
+    return KIND == EPI_GATEUP ? ru * 256 + half * 128 : ru * 512 + half * 256;
   };
 
   if (warp < 4) {
@@ -402,33 +401,26 @@ __global__ void __launch_bounds__(kWThreads, 1)
       auto advance = [&](Pos& p) {
         if (++p.k == p.sg.k1) seek(p);
       };
-      auto box = [&](const CUtensorMap* m, uint8_t* dst, uint64_t* bar, int x, int y) {
-        if constexpr (kPairs == 1) tma_load_2d_pair(dst, m, bar, x, y);
-        else tma_load_2d_pair_mc(dst, m, bar, x, y, static_cast<uint16_t>(5u << r));
-      };
       const int half = e.hd >> 1;
-      // this CTA's weight tiles of a chunk: both, or with two pairs the one it
-      // loads for both (accumulator 0's rows by pair 0)
       auto load_a = [&](const Pos& p, int st) {
         uint64_t* bar = &s.full[st];
         const int x = p.k * kBK;
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
-          if (kPairs == 2 && a != pair) continue;
           uint8_t* dst = ring + st * kWStage + a * kWATile;
           if constexpr (KIND == EPI_GATEUP) {
             const CUtensorMap* m = a == 0 ? &mA0 : &mA1;
-            box(m, dst, bar, x, p.row0);
-            box(m, dst + kWATile / 2, bar, x, p.row0 + 64);
+            tma_load_2d_pair(dst, m, bar, x, p.row0);
+            tma_load_2d_pair(dst + kWATile / 2, m, bar, x, p.row0 + 64);
           } else if constexpr (KIND == EPI_QKV) {
             for (int i = 0, y = p.row0 + a * half; i < kBM; i += half, y += e.hd) {
               uint8_t* d = dst + i * kBK * 2;
-              if (y < g.rows_q) box(&mA0, d, bar, x, y);
-              else if (y < g.rows_qk) box(&mA1, d, bar, x, y - g.rows_q);
-              else box(&mA2, d, bar, x, y - g.rows_qk);  // (past V: the map's zero fill)
+              if (y < g.rows_q) tma_load_2d_pair(d, &mA0, bar, x, y);
+              else if (y < g.rows_qk) tma_load_2d_pair(d, &mA1, bar, x, y - g.rows_q);
+              else tma_load_2d_pair(d, &mA2, bar, x, y - g.rows_qk);  // (past V: the map's zero fill)
             }
           } else {
-            box(&mA0, dst, bar, x, p.row0 + a * kBM);
+            tma_load_2d_pair(dst, &mA0, bar, x, p.row0 + a * kBM);
           }
         }
       };
@@ -466,7 +458,6 @@ __global__ void __launch_bounds__(kWThreads, 1)
     }
     if (warp == 1 && lane == 0 && leader) {
       const uint32_t idesc = idesc_bf16_f32(256, 2 * g.bn);
-      const uint16_t pair_mask = static_cast<uint16_t>(3u << (2 * pair));
       uint32_t accph = 0;
       int idx = 0;
       bool ok = true;
@@ -487,13 +478,13 @@ __global__ void __launch_bounds__(kWThreads, 1)
             for (int kk = 0; kk < kBK / 16; ++kk)
               tc_mma_f16_pair(tmem + a * 256, sdesc_kmajor_sw128(a_addr + a * kWATile + kk * 32),
                               sdesc_kmajor_sw128(b_addr + kk * 32), idesc, (k > sg.k0 || kk > 0) ? 1u : 0u);
-          tc_commit_pair(&s.empty[st], kAllMask);
+          tc_commit_pair(&s.empty[st], 3);
         }
-        if (ok) tc_commit_pair(&s.tfull, pair_mask);
+        if (ok) tc_commit_pair(&s.tfull, 3);
         accph ^= 1;
       }
       // every issued MMA has completed (bounded)
-      tc_commit_pair(&s.drain, static_cast<uint16_t>(1u << crank));
+      tc_commit_pair(&s.drain, 1);
       mbar_wait(&s.drain, 0, nullptr);
     }
   } else {
@@ -503,7 +494,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
     const int grp = et >> 7;             // token chunks grp, grp + 2, ...
     const int lr = (warp & 3) * 32 + lane;  // tensor-memory lane = row of a weight tile
     const uint32_t taddr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-    const uint32_t tempty_leader = mapa_smem(&s.tempty, crank & ~1u);
+    const uint32_t tempty_leader = mapa_smem(&s.tempty, 0);
     auto joint = [&]() { named_bar_sync(3, 256); };
     uint32_t accph = 0;
     while (work.next(sg, cluster, first, last)) {
@@ -545,7 +536,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_remote(tempty_leader);  // the next unit's MMAs may start
       if (!owner) {
-        float* part = g.partial + (static_cast<size_t>(cluster) * kCl + crank) * kWidePartFloats;
+        float* part = g.partial + (static_cast<size_t>(cluster) * 2 + r) * kWidePartFloats;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           if ((grp + 2 * q) * kEpiCols < g.bn) {
@@ -554,15 +545,15 @@ __global__ void __launch_bounds__(kWThreads, 1)
           }
         }
         joint();  // every thread's stores precede the release
-        if (et == 0) red_release_gpu(&g.tickets[first * kCl + crank], 1);
+        if (et == 0) red_release_gpu(&g.tickets[first * 2 + r], 1);
         continue;
       }
       if (last > first) {
-        if (et == 0) s.ok[1] = count_wait(&g.tickets[first * kCl + crank], last - first, abort) ? 1 : 0;
+        if (et == 0) s.ok[1] = count_wait(&g.tickets[first * 2 + r], last - first, abort) ? 1 : 0;
         joint();
         if (!s.ok[1]) break;
         for (int o = first + 1; o <= last; ++o) {
-          const float* part = g.partial + (static_cast<size_t>(o) * kCl + crank) * kWidePartFloats;
+          const float* part = g.partial + (static_cast<size_t>(o) * 2 + r) * kWidePartFloats;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             if ((grp + 2 * q) * kEpiCols < g.bn) {
@@ -571,7 +562,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
             }
           }
         }
-        if (et == 0) g.tickets[first * kCl + crank] = 0;
+        if (et == 0) g.tickets[first * 2 + r] = 0;
       }
       wide_apply<KIND>(e, g, row0, t0, lr, grp, v0, v1, s);
       joint();  // the tables are rewritten for the next unit
@@ -619,45 +610,44 @@ __global__ void __launch_bounds__(128) argmax_reduce_kernel(const EpiArgs e) {
 
 // ---- launchers ----------------------------------------------------------------------
 
-template <int KIND, int CL>
+template <int KIND>
 static cudaError_t wide_set_one() {
-  return cudaFuncSetAttribute(gemm_wide_kernel<KIND, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(gemm_wide_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(wide_smem_bytes()));
 }
 
-cudaError_t gemm_wide_set_attributes_acc() { return wide_set_one<EPI_ACC, kWideCluster>(); }
+cudaError_t gemm_wide_set_attributes_acc() { return wide_set_one<EPI_ACC>(); }
 
 cudaError_t gemm_wide_set_attributes() {
   cudaError_t err;
-  if ((err = wide_set_one<EPI_QKV, kWideCluster>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_GATEUP, kWideCluster>()) != cudaSuccess) return err;
-  if ((err = wide_set_one<EPI_RESID, kWideCluster>()) != cudaSuccess) return err;
-  return wide_set_one<EPI_ARGMAX, kWideCluster>();
+  if ((err = wide_set_one<EPI_QKV>()) != cudaSuccess) return err;
+  if ((err = wide_set_one<EPI_GATEUP>()) != cudaSuccess) return err;
+  if ((err = wide_set_one<EPI_RESID>()) != cudaSuccess) return err;
+  return wide_set_one<EPI_ARGMAX>();
 }
 
 // Clusters that can be resident at once (0: none, or an error).
 int gemm_wide_clusters() {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
-  cfg.gridDim = dim3(kWideCluster * 64);
+  cfg.gridDim = dim3(2 * 64);
   cfg.blockDim = dim3(kWThreads);
   cfg.dynamicSmemBytes = wide_smem_bytes();
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kWideCluster;
+  attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  return cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI_ACC, kWideCluster>, &cfg) == cudaSuccess ? n : 0;
+  return cudaOccupancyMaxActiveClusters(&n, gemm_wide_kernel<EPI_ACC>, &cfg) == cudaSuccess ? n : 0;
 }
 
 WidePlan plan_wide(int kind, int M, int K, int T, int clusters, bool split) {
   WidePlan p{};
-  constexpr int pairs = kWideCluster / 2;
   p.row_units = ceil_div(M, kind == EPI_GATEUP ? 256 : 512);
-  p.ntiles = ceil_div(T, kWideTokens * pairs);
-  p.bn = round_up(ceil_div(T, p.ntiles * pairs), kEpiCols);
+  p.ntiles = ceil_div(T, kWideTokens);
+  p.bn = round_up(ceil_div(T, p.ntiles), kEpiCols);
   p.kchunks = ceil_div(K, kBK);
   const int units = p.row_units * p.ntiles, rest = units % clusters;
   p.cpc = split ? std::max(1, ceil_div(rest * p.kchunks, clusters)) : p.kchunks;
@@ -666,38 +656,38 @@ WidePlan plan_wide(int kind, int M, int K, int T, int clusters, bool split) {
   return p;
 }
 
-template <int KIND, int CL>
+template <int KIND>
 static cudaError_t launch_wide_one(const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
                                    cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[2];
-  cfg.gridDim = dim3(clusters * CL);
+  cfg.gridDim = dim3(clusters * 2);
   cfg.blockDim = dim3(kWThreads);
   cfg.dynamicSmemBytes = wide_smem_bytes();
   cfg.stream = s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<KIND, CL>, m.a0, m.a1, m.a2, m.b, g, e);
+  return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<KIND>, m.a0, m.a1, m.a2, m.b, g, e);
 }
 
 cudaError_t launch_gemm_wide(int kind, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int clusters,
                              cudaStream_t s, bool pdl) {
   cudaError_t err;
   switch (kind) {
-    case EPI_QKV: return launch_wide_one<EPI_QKV, kWideCluster>(m, g, e, clusters, s, pdl);
-    case EPI_GATEUP: return launch_wide_one<EPI_GATEUP, kWideCluster>(m, g, e, clusters, s, pdl);
-    case EPI_RESID: return launch_wide_one<EPI_RESID, kWideCluster>(m, g, e, clusters, s, pdl);
-    case EPI_ACC: return launch_wide_one<EPI_ACC, kWideCluster>(m, g, e, clusters, s, pdl);
+    case EPI_QKV: return launch_wide_one<EPI_QKV>(m, g, e, clusters, s, pdl);
+    case EPI_GATEUP: return launch_wide_one<EPI_GATEUP>(m, g, e, clusters, s, pdl);
+    case EPI_RESID: return launch_wide_one<EPI_RESID>(m, g, e, clusters, s, pdl);
+    case EPI_ACC: return launch_wide_one<EPI_ACC>(m, g, e, clusters, s, pdl);
     case EPI_ARGMAX: break;
     default: return cudaErrorInvalidValue;
   }
-  if ((err = launch_wide_one<EPI_ARGMAX, kWideCluster>(m, g, e, clusters, s, pdl)) != cudaSuccess) return err;
+  if ((err = launch_wide_one<EPI_ARGMAX>(m, g, e, clusters, s, pdl)) != cudaSuccess) return err;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
   cfg.gridDim = dim3((e.T + 15) / 16);

@@ -312,7 +312,6 @@ inline int pair_box_rows(int bn) { return bn <= 128 ? bn : bn / 2; }
 // of cpc chunks per cluster.
 constexpr int kWideTokens = 128;                     // most tokens of a pair's tile
 constexpr int kWidePartFloats = 2 * kWideTokens * kBM;  // a CTA's split-K partial
-constexpr int kWideCluster = 4;                      // CTAs per cluster
 struct WidePlan {
   int row_units, ntiles, bn, kchunks, cpc, clusters;
   void apply(GemmArgs& g) const {
