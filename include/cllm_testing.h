@@ -114,6 +114,17 @@ int cllm_test_plan_gemm(int mtiles, int K, int T, int sms, int *out);
  */
 int cllm_test_plan_group(int mtiles, int K, int T, int sms, int *out);
 
+/*
+ * Host-only: the work split of a launch of more than 256 tokens over `clusters`
+ * CTA pairs (any T >= 1 is planned).  out[6] = {row units (512 weight rows;
+ * gate_up: 256 features), token tiles, tokens per tile, kchunks, cpc, clusters
+ * launched}.  Unit u = row unit * token tiles + token tile.  Clusters take
+ * units u = cluster, cluster + clusters, ... for as many whole rounds as there
+ * are; the (unit, chunk) space of the rest is cut into ranges of cpc chunks.
+ * split 0: ranges are whole units.  EINVAL as above.
+ */
+int cllm_test_plan_wide(int gate_up, int M, int K, int T, int clusters, int split, int *out);
+
 #ifdef __cplusplus
 }
 #endif

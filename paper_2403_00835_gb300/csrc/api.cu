@@ -172,7 +172,7 @@ struct cllm_ctx {
   size_t gemm_part_elems = 0;
   int* tickets = nullptr;
   int wide_clusters = 0;       // wide GEMM launches: resident clusters
-  float* wide_part = nullptr;          // one split-K partial per CTA
+  float* wide_part = nullptr;  // two split-K partials per CTA
   int* wide_tickets = nullptr;
   int max_mtiles = 0;
   float* am_part = nullptr;
@@ -1366,7 +1366,7 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
     c->gemm_part_elems = need;
     if (c->bf16 && c->Tcap > 256) {
       const size_t ctas = static_cast<size_t>(c->wide_clusters) * 2;
-      ok = ok && dev_alloc(c, &c->wide_part, ctas * kWidePartFloats * 4) && dev_alloc(c, &c->wide_tickets, ctas * 4);
+      ok = ok && dev_alloc(c, &c->wide_part, 2 * ctas * kWidePartFloats * 4) && dev_alloc(c, &c->wide_tickets, ctas * 4);
     }
     ok = ok && dev_alloc(c, &c->gemm_part, need * 4) && dev_alloc(c, &c->tickets, c->max_mtiles * 4) &&
          dev_alloc(c, &c->am_part, static_cast<size_t>(ceil_div(c->V, kBM)) * T * 12) &&
@@ -1957,7 +1957,7 @@ extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M
   do {
     const size_t ctas = static_cast<size_t>(w.clusters) * 2;
     float* part = static_cast<float*>(
-        alloc(wide ? ctas * kWidePartFloats * 4 : static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
+        alloc(wide ? 2 * ctas * kWidePartFloats * 4 : static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
     int* tickets = static_cast<int*>(alloc(wide ? ctas * 4 : mtiles * 4));
     int* err = static_cast<int*>(alloc(16));
     float* ssq = static_cast<float*>(alloc(static_cast<size_t>(mtiles) * ldt * 4));
@@ -2182,6 +2182,14 @@ extern "C" int cllm_test_plan_group(int mtiles, int K, int T, int sms, int* out)
   if (!out || mtiles < 1 || K < 1 || T < 1 || T > 256 || sms < 1) return CLLM_EINVAL;
   const Part p = plan_group(mtiles, K, T, sms);
   const int v[8] = {p.mtiles, 1 << kGroupShift, p.kchunks, p.cpc, p.bn, p.bn_max, p.maxc, p.grid};
+  std::memcpy(out, v, sizeof v);
+  return CLLM_OK;
+}
+
+extern "C" int cllm_test_plan_wide(int gate_up, int M, int K, int T, int clusters, int split, int* out) {
+  if (!out || M < 1 || K < 1 || T < 1 || clusters < 1) return CLLM_EINVAL;
+  const WidePlan p = plan_wide(gate_up ? EPI_GATEUP : EPI_RESID, M, K, T, clusters, split != 0);
+  const int v[6] = {p.row_units, p.ntiles, p.bn, p.kchunks, p.cpc, p.clusters};
   std::memcpy(out, v, sizeof v);
   return CLLM_OK;
 }

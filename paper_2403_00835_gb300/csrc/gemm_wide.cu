@@ -23,10 +23,15 @@
 // clusters working at one time share weights through L2) goes to cluster
 // u mod clusters for as many whole rounds as there are; the remaining units'
 // (unit, K chunk) space is cut into equal contiguous ranges, one per cluster.
-// A range's first segment may be the end of a unit that an earlier cluster
-// began: its sums go to a global partial, and the unit's first contributor
-// (for which it is the last segment) adds the partials in range order, so the
-// result does not depend on timing.
+// A unit cut over several ranges is finished by whichever contributor is the
+// last to arrive (a ticket); the others leave their sums in global partials.
+// No cluster ever waits for another one, so the launch needs no co-residency
+// (another engine's launches may hold part of the SMs), and the sums are added
+// in range order, so the result does not depend on the order of arrival.
+// (The first contributor waiting for the others saved the store of its own
+// sums -- 500 rows 1.25 against 1.29 ms, 4096 rows 5.53 against 5.58 -- but two
+// engines' launches, each with part of its clusters resident, could hold each
+// other until the waits ran out.)
 //
 // Per launch at 2048 rows, 7B shape, against the single-CTA kernel: gate/up
 // 757 -> 384 us (1.93 PFLOP/s counting both planes: the power limit), QKV 555
@@ -71,7 +76,7 @@ struct WideSmem {
   uint64_t full[kWStages], empty[kWStages], tfull, tempty, drain;
   uint32_t tmem;
   int abort_flag;
-  int ok[2];  // [0] the accumulator wait's result, [1] the split-K wait's
+  int ok[2];  // [0] the accumulator wait's result, [1] this cluster finishes the unit
 };
 
 constexpr size_t wide_smem_bytes() { return 1024 + kWStages * kWStage + sizeof(WideSmem); }
@@ -499,8 +504,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
     uint32_t accph = 0;
     while (work.next(sg, cluster, first, last)) {
       const int t0 = unit_tok(sg.unit), row0 = unit_row(sg.unit);
-      const bool owner = cluster == first;
-      if (owner && KIND != EPI_RESID && KIND != EPI_ACC) {
+      if (KIND != EPI_RESID && KIND != EPI_ACC) {
         // the unit's RMSNorm scales, positions and sequences, while its MMAs run
         const int tq = (et >> 3) * 4, part = et & 7;
         if ((et & ~31) / 2 < g.bn) {  // (a warp's 4 column quads; bn is a multiple of 16)
@@ -535,25 +539,45 @@ __global__ void __launch_bounds__(kWThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_remote(tempty_leader);  // the next unit's MMAs may start
-      if (!owner) {
-        float* part = g.partial + (static_cast<size_t>(cluster) * 2 + r) * kWidePartFloats;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if ((grp + 2 * q) * kEpiCols < g.bn) {
-            part_st16(part, grp + 2 * q, lr, v0[q]);
-            part_st16(part, 8 + grp + 2 * q, lr, v1[q]);
-          }
-        }
-        joint();  // every thread's stores precede the release
-        if (et == 0) red_release_gpu(&g.tickets[first * 2 + r], 1);
-        continue;
-      }
       if (last > first) {
-        if (et == 0) s.ok[1] = count_wait(&g.tickets[first * 2 + r], last - first, abort) ? 1 : 0;
+        // A cluster has at most two cut segments, one that begins its unit and
+        // one that does not, with a partial slot each.
+        int* ticket = &g.tickets[first * 2 + r];
+        auto part_of = [&](int o) {
+          return g.partial + (static_cast<size_t>(o * 2 + (o == first)) * 2 + r) * kWidePartFloats;
+        };
+        // The sums are added in range order.  The first two contributors may
+        // add the others' to their registers (a + b = b + a); a later one starts
+        // again from the partials, its own among them.
+        const bool reload = cluster > first + 1;
+        // (all the others' sums may be there already: no need to store)
+        if (et == 0)
+          s.ok[1] = !reload && static_cast<int>(ld_acquire_gpu(reinterpret_cast<unsigned*>(ticket))) == last - first;
         joint();
-        if (!s.ok[1]) break;
-        for (int o = first + 1; o <= last; ++o) {
-          const float* part = g.partial + (static_cast<size_t>(o) * 2 + r) * kWidePartFloats;
+        if (!s.ok[1]) {
+          float* part = part_of(cluster);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if ((grp + 2 * q) * kEpiCols < g.bn) {
+              part_st16(part, grp + 2 * q, lr, v0[q]);
+              part_st16(part, 8 + grp + 2 * q, lr, v1[q]);
+            }
+          }
+          joint();  // every thread's stores precede the arrival
+          if (et == 0) s.ok[1] = ticket_add(ticket, 1) == last - first;
+          joint();
+          if (!s.ok[1]) continue;
+        }
+        if (et == 0) *ticket = 0;
+        if (reload) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int j = 0; j < kEpiCols; ++j) v0[q][j] = v1[q][j] = 0.f;
+        }
+        for (int o = first; o <= last; ++o) {
+          if (o == cluster && !reload) continue;
+          const float* part = part_of(o);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             if ((grp + 2 * q) * kEpiCols < g.bn) {
@@ -562,7 +586,6 @@ __global__ void __launch_bounds__(kWThreads, 1)
             }
           }
         }
-        if (et == 0) g.tickets[first * 2 + r] = 0;
       }
       wide_apply<KIND>(e, g, row0, t0, lr, grp, v0, v1, s);
       joint();  // the tables are rewritten for the next unit

@@ -311,7 +311,7 @@ inline int pair_box_rows(int bn) { return bn <= 128 ? bn : bn / 2; }
 // 256 features) x bn tokens per CTA pair, the (unit, K chunk) space in ranges
 // of cpc chunks per cluster.
 constexpr int kWideTokens = 128;                     // most tokens of a pair's tile
-constexpr int kWidePartFloats = 2 * kWideTokens * kBM;  // a CTA's split-K partial
+constexpr int kWidePartFloats = 2 * kWideTokens * kBM;  // one split-K partial (a CTA may leave two)
 struct WidePlan {
   int row_units, ntiles, bn, kchunks, cpc, clusters;
   void apply(GemmArgs& g) const {
@@ -322,8 +322,8 @@ struct WidePlan {
     g.cpc = cpc;
   }
 };
-// split: ranges may cut a unit (needs kWidePartFloats floats and one zeroed
-// ticket per CTA); otherwise whole units
+// split: ranges may cut a unit (needs two partials and one zeroed ticket per
+// CTA); otherwise whole units
 WidePlan plan_wide(int kind, int M, int K, int T, int clusters, bool split);
 int gemm_wide_clusters();  // after the attributes of the EPI_ACC kernel are set
 cudaError_t gemm_wide_set_attributes();

@@ -53,6 +53,36 @@ def test_wide_gemm_matches_fp64(M, K, T, noalloc):
     assert bool(((Y.double() - ref).abs() <= bound).all())
 
 
+@pytest.mark.parametrize("M,K,T", [(4096, 4096, 300), (1024, 11008, 257), (512, 688, 400), (12288, 4096, 500)])
+def test_wide_gemm_bits_do_not_depend_on_the_order_of_arrival(M, K, T):
+    """Units cut over several pairs are finished by the last contributor; the
+    sums are added in range order whoever that is.  Products of another stream
+    hold SMs meanwhile, so that pairs start late and finish out of order."""
+    lib = cllm.load()
+    lib.cllm_test_gemm_bf16.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int] * 4
+    g = torch.Generator(device="cuda").manual_seed(M + K + T)
+    W = (torch.randn(M, K, device="cuda", generator=g) * 0.02).bfloat16()
+    rows = (T + 15) // 16 * 16
+    x = torch.randn(rows, K, device="cuda", generator=g)
+    hi = x.bfloat16()
+    X2 = torch.stack([hi, (x - hi.float()).bfloat16()]).contiguous()
+    noise = torch.randn(2048, 2048, device="cuda", generator=g).bfloat16()
+    other = torch.cuda.Stream()
+    outs = []
+    for busy in (False, True, True, True, False):
+        Y = torch.zeros(T, M, device="cuda")
+        torch.cuda.synchronize()
+        if busy:
+            with torch.cuda.stream(other):
+                for _ in range(200):
+                    noise @ noise
+        assert lib.cllm_test_gemm_bf16(W.data_ptr(), X2.data_ptr(), Y.data_ptr(), M, K, T, rows) == 0
+        torch.cuda.synchronize()
+        outs.append(Y)
+    for Y in outs[1:]:
+        assert torch.equal(Y, outs[0])
+
+
 @pytest.mark.parametrize("hd,kv,ffn,lens", [
     (64, 4, 688, [300]), (64, 2, 264, [150, 200, 7]), (128, 1, 688, [257]), (128, 2, 520, [100, 420])])
 def test_wide_prefill_matches_oracle(hd, kv, ffn, lens):
