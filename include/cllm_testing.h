@@ -85,6 +85,17 @@ int cllm_test_set_trace_phase(cllm_ctx *ctx, int phase);
 int cllm_test_hold_barrier(cllm_ctx *ctx, int phase);
 
 /*
+ * The same for the split-K waits of launches of up to 256 rows: every weight
+ * tile's arrival count is set to `count`.  With -1 the first contributor of a
+ * tile that is cut over several ranges waits for one arrival more than there
+ * are; its wait runs out (2 s), the launch ends and the call that ran it
+ * returns CLLM_ETIMEOUT.  The counts are left as the launches leave them, so
+ * the context stays usable only if the library resets them.  EINVAL on a null
+ * ctx.
+ */
+int cllm_test_arm_splits(cllm_ctx *ctx, int count);
+
+/*
  * Allocation-failure injection: the k-th device (or pinned host) allocation
  * the library makes from now on (k = 0: the next one) fails as if memory
  * were exhausted; the call that made it returns CLLM_ENOMEM after releasing

@@ -222,6 +222,8 @@ struct cllm_ctx {
     unsigned long long* stamps = nullptr;
     unsigned long long* cta_stamps = nullptr;
     size_t bar_bytes = 64;             // grid-barrier counter and completion flags
+    int* attn_tickets = nullptr;       // ranges done per (query tile, head)
+    size_t attn_ticket_bytes = 0;
   };
   // one persistent kernel per iteration: -1 where it is faster, 1 wherever it is
   // supported, 0 never
@@ -631,6 +633,29 @@ AcceptArgs make_accept(cllm_ctx* c, int B, int n, bool decode) {
   return a;
 }
 
+// Clear a device error that the host has read and map it to a status.  The
+// launches' arrival counters go back to zero by themselves only while no wait
+// runs out: after a timeout some hold the arrivals of an unfinished tile, and
+// the next launch would take its own first partials for all of them.  The
+// memsets follow whatever is still queued on the stream.
+int clear_device_error(cllm_ctx* c, int e) {
+  bool ok = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) == cudaSuccess;
+  if (e & DERR_TIMEOUT) {
+    auto zero = [&](void* p, size_t bytes) {
+      if (p) ok = cudaMemsetAsync(p, 0, bytes, c->stream) == cudaSuccess && ok;
+    };
+    zero(c->tickets, static_cast<size_t>(c->max_mtiles) * 4);
+    zero(c->wide_tickets, static_cast<size_t>(c->wide_clusters) * 2 * 4);
+    zero(c->attn_tickets, static_cast<size_t>(c->max_qtiles) * c->H * 4);
+    zero(c->am_ticket, 16);
+    for (auto& kv : c->graphs) zero(kv.second.attn_tickets, kv.second.attn_ticket_bytes);
+  }
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess || !ok) return cuda_fail(cudaGetLastError(), "error reset");
+  if (e & DERR_TIMEOUT) return CLLM_ETIMEOUT;
+  if (e & DERR_CAPACITY) return CLLM_ECAPACITY;
+  return CLLM_EDEVICE;
+}
+
 // Read the device status (active, committed, error) after a synchronisation.
 int check_device_error(cllm_ctx* c) {
   int e = 0;
@@ -640,12 +665,7 @@ int check_device_error(cllm_ctx* c) {
   ce = cudaStreamSynchronize(c->stream);
   if (ce != cudaSuccess) return cuda_fail(ce, "stream sync");
   e = c->status_host[2];
-  if (e == 0) return CLLM_OK;
-  cudaMemsetAsync(c->err, 0, sizeof(int), c->stream);
-  cudaStreamSynchronize(c->stream);
-  if (e & DERR_TIMEOUT) return CLLM_ETIMEOUT;
-  if (e & DERR_CAPACITY) return CLLM_ECAPACITY;
-  return CLLM_EDEVICE;
+  return e == 0 ? CLLM_OK : clear_device_error(c, e);
 }
 
 std::vector<int2> step_qtiles(int B, int n) {
@@ -845,7 +865,8 @@ int build_persistent(cllm_ctx* c, int mode, int B, int n, const int2* qtiles, in
   if (maps.size() > static_cast<size_t>(kMaxStepMaps)) return CLLM_EUNSUPPORTED;
   for (size_t i = 0; i < maps.size(); ++i) prm.maps[i] = maps[i];
   void* ph_d = upload(ph.data(), ph.size() * sizeof(PhaseDesc));
-  void* tk_d = upload(nullptr, static_cast<size_t>(n_qtiles) * c->H * sizeof(int) + 16);
+  ge.attn_ticket_bytes = static_cast<size_t>(n_qtiles) * c->H * sizeof(int) + 16;
+  void* tk_d = upload(nullptr, ge.attn_ticket_bytes);
   void* st_d = upload(nullptr, (5 * ph.size() + 1) * sizeof(unsigned long long));
   void* cst_d = upload(nullptr, (kCtaStampSlots * ph.size() + kTraceCap) * c->sms *
                                     sizeof(unsigned long long));
@@ -871,7 +892,7 @@ int build_persistent(cllm_ctx* c, int mode, int B, int n, const int2* qtiles, in
   sa.bar = static_cast<unsigned*>(bar_d);
   sa.embed = make_embed_args(c, f);
   sa.attn = make_attn_args(c, f);
-  sa.attn_tickets = static_cast<int*>(tk_d);
+  sa.attn_tickets = ge.attn_tickets = static_cast<int*>(tk_d);
   sa.accept = make_accept(c, B, n, mode == MODE_DECODE);
   sa.stamps = c->profiling ? ge.stamps : nullptr;
   sa.cta_stamps = c->profiling ? ge.cta_stamps : nullptr;
@@ -1129,12 +1150,7 @@ void accumulate_profile(cllm_ctx* c, const cllm_ctx::GraphEntry* ge) {
 
 int read_status(cllm_ctx* c, int slot) {
   const int e = c->status_host[4 * slot + 2];
-  if (e == 0) return CLLM_OK;
-  cudaMemsetAsync(c->err, 0, sizeof(int), c->stream);
-  cudaStreamSynchronize(c->stream);
-  if (e & DERR_TIMEOUT) return CLLM_ETIMEOUT;
-  if (e & DERR_CAPACITY) return CLLM_ECAPACITY;
-  return CLLM_EDEVICE;
+  return e == 0 ? CLLM_OK : clear_device_error(c, e);
 }
 
 }  // namespace
@@ -2166,6 +2182,16 @@ extern "C" int cllm_test_hold_barrier(cllm_ctx* c, int phase) {
   if (!c || phase == 0 || phase < -1) return CLLM_EINVAL;
   c->hold_phase = phase;
   return drop_graphs(c);
+}
+
+extern "C" int cllm_test_arm_splits(cllm_ctx* c, int count) {
+  if (!c) return CLLM_EINVAL;
+  cudaSetDevice(c->dev);
+  const std::vector<int> v(c->max_mtiles, count);
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess ||
+      cudaMemcpy(c->tickets, v.data(), v.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
+    return cuda_fail(cudaGetLastError(), "arm splits");
+  return CLLM_OK;
 }
 
 extern "C" void cllm_test_fail_alloc(int k) { g_alloc_countdown.store(k < 0 ? -1 : k); }

@@ -5,6 +5,8 @@
     runs out after the wait budget, the kernel unwinds (copies and
     tensor-core work in flight are waited for, tensor memory is freed), the
     call returns CLLM_ETIMEOUT, and the context decodes correctly afterwards;
+  * a split-K wait that runs out leaves no arrival counts behind: the next
+    calls return what a context that never timed out returns;
   * allocation failure: a countdown makes the k-th device or pinned
     allocation fail; the call returns CLLM_ENOMEM, releases what it had taken
     and leaves the process able to create and run a context.
@@ -89,6 +91,37 @@ def test_hold_barrier_rejects_bad_phase(tiny):
         assert lib.cllm_test_hold_barrier(eng._h, 0) == -1
         assert lib.cllm_test_hold_barrier(eng._h, -2) == -1
         assert lib.cllm_test_hold_barrier(None, 1) == -1
+    finally:
+        eng.close()
+
+
+@pytest.mark.parametrize("rows", [64, 16])
+def test_split_timeout_leaves_no_counts_behind(tiny, rows):
+    """The down projection's tiles (K = 688) are cut over three ranges.  One
+    prefill's waits run out there (per-phase launches), or one step's in the
+    persistent kernel; afterwards every tile must again wait for all of its
+    contributors, so the logits have a fresh context's bits."""
+    cfg, w = tiny
+    lib = _hooks()
+    lib.cllm_test_arm_splits.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.cllm_test_arm_splits.restype = ctypes.c_int
+    assert lib.cllm_test_arm_splits(None, -1) == -1
+    prompts = syn.make_prompts(cfg.vocab, [rows], seed=83)
+    guesses = syn.make_guesses(cfg.vocab, 1, rows, seed=84)
+    eng = engine_for(cfg, w, max_batch=1, max_seq=3 * rows, max_block=rows)
+    try:
+        head = eng.prefill(prompts)
+        ref = eng.jacobi_step(guesses, want_logits=True)
+        assert eng.uses_persistent(rows) == (rows < 64)
+        for call in ("prefill", "step"):
+            eng.prefill(prompts)
+            assert lib.cllm_test_arm_splits(eng._h, -1) == 0
+            with pytest.raises(CllmError) as e:
+                eng.prefill(prompts) if call == "prefill" else eng.jacobi_step(guesses)
+            assert e.value.status == CLLM_ETIMEOUT, call
+            np.testing.assert_array_equal(eng.prefill(prompts), head)
+            r = eng.jacobi_step(guesses, want_logits=True)
+            np.testing.assert_array_equal(r["logits"], ref["logits"])
     finally:
         eng.close()
 
