@@ -85,6 +85,16 @@ int cllm_test_set_trace_phase(cllm_ctx *ctx, int phase);
 int cllm_test_hold_barrier(cllm_ctx *ctx, int phase);
 
 /*
+ * The same for the attention of launches with many rows per sequence: the
+ * thread that issues its tensor-core work stops before key chunk `chunk` >= 0,
+ * as if its own wait had run out.  The softmax warps' waits run out (2 s), the
+ * CTA waits for its loads and tensor-core operations in flight, frees its
+ * tensor memory and returns, and the call returns CLLM_ETIMEOUT.  -1 disarms.
+ * Drops the captured graphs.  EINVAL on a null ctx or chunk < -1.
+ */
+int cllm_test_hold_attention(cllm_ctx *ctx, int chunk);
+
+/*
  * The same for the split-K waits of launches of up to 256 rows: every weight
  * tile's arrival count is set to `count`.  With -1 the first contributor of a
  * tile that is cut over several ranges waits for one arrival more than there

@@ -236,6 +236,7 @@ struct cllm_ctx {
   std::vector<unsigned long long> last_cta_stamps;
   int trace_phase = -1;  // profiling: phase whose MMA stage arrivals are traced
   int hold_phase = -1;   // test hook: grid barrier that cannot open (bounded-wait path)
+  int hold_attn = 0;     // test hook: 1 + the chunk at which the wide attention stops
   bool step_logits = false;  // the step graph being built stores the LM head's logits
   std::map<std::tuple<int, int, int, int, int, unsigned long long, int, int, int, int>, GraphEntry>
       graphs;
@@ -497,6 +498,7 @@ cudaError_t record_forward(cllm_ctx* c, cudaStream_t s, const FwdSpec& f, bool p
   AttnArgs aw = aa;  // wide attention
   aw.qtiles = f.wtiles;
   aw.n_qtiles = f.n_wtiles;
+  aw.hold = c->hold_attn;
 
   for (int l = 0; l < c->NL; ++l) {
     const LayerW& L = c->layers[l];
@@ -2181,6 +2183,12 @@ extern "C" int cllm_test_set_trace_phase(cllm_ctx* c, int phase) {
 extern "C" int cllm_test_hold_barrier(cllm_ctx* c, int phase) {
   if (!c || phase == 0 || phase < -1) return CLLM_EINVAL;
   c->hold_phase = phase;
+  return drop_graphs(c);
+}
+
+extern "C" int cllm_test_hold_attention(cllm_ctx* c, int chunk) {
+  if (!c || chunk < -1) return CLLM_EINVAL;
+  c->hold_attn = chunk + 1;
   return drop_graphs(c);
 }
 

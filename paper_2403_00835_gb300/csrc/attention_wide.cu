@@ -41,7 +41,7 @@ struct WideAttnSmem {
   alignas(1024) uint8_t q[2][kWQ * HD * 2];
   alignas(1024) uint8_t k[2][kAttnChunk * HD * 2];
   alignas(1024) uint8_t v[2][kAttnChunk * HD * 2];
-  uint64_t qfull, kfull[2], vfull[2], sfull[2], pready[2], ofull[2];
+  uint64_t qfull, kfull[2], vfull[2], sfull[2], pready[2], ofull[2], drain;
   uint32_t tmem;
   int abort_flag;
 };
@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(kWAttnThreads, 1)
   volatile int* abort = &s.abort_flag;
   if (threadIdx.x == 0) {
     mbar_init(&s.qfull, 1);
+    mbar_init(&s.drain, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s.kfull[i], 1);
       mbar_init(&s.vfull[i], 1);
@@ -152,6 +153,10 @@ __global__ void __launch_bounds__(kWAttnThreads, 1)
       }
       for (int c = 0; ok && c < n; ++c) {
         const int nt[2] = {n0, n1};
+        if (a.hold == c + 1) {  // test hook: as if this thread's wait had run out
+          ok = false;
+          break;
+        }
         ok = mbar_wait(&s.vfull[c & 1], (c >> 1) & 1, abort);
         if (ok && c + 1 < n) ok = mbar_wait(&s.kfull[(c + 1) & 1], ((c + 1) >> 1) & 1, abort);
 #pragma unroll
@@ -178,7 +183,10 @@ __global__ void __launch_bounds__(kWAttnThreads, 1)
         }
       }
       if (!ok) {
-        // loads in flight land (bounded) before the CTA leaves
+        // MMAs and loads in flight end (bounded) before the CTA leaves (otherwise
+        // the tiles' last commits, which the softmax warps wait for, cover them)
+        tc_commit(&s.drain);
+        mbar_wait(&s.drain, 0, nullptr);
         mbar_wait(&s.qfull, 0, nullptr);
         for (int c = max(0, loads_k - 2); c < loads_k; ++c) mbar_wait(&s.kfull[c & 1], (c >> 1) & 1, nullptr);
         for (int c = max(0, loads_v - 2); c < loads_v; ++c) mbar_wait(&s.vfull[c & 1], (c >> 1) & 1, nullptr);
@@ -192,14 +200,22 @@ __global__ void __launch_bounds__(kWAttnThreads, 1)
     const int p_row = pos0 + t * kWQ + row;  // this row's position: it sees keys 0..p_row
     const int p_first = pos0 + t * kWQ;
     const uint32_t ts = tmem + t * 256 + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    // (one lane waits for its warp: lanes that gave up on their own would leave
+    // the others at a warp-wide operation)
+    auto warp_wait = [&](uint64_t* bar, uint32_t parity) {
+      int got = 0;
+      if (lane == 0) got = mbar_wait(bar, parity, abort) ? 1 : 0;
+      got = __shfl_sync(0xffffffffu, got, 0);
+      __syncwarp();
+      return got != 0;
+    };
     float mx = -INFINITY, l = 0.f;
     bool ok = true;
     for (int c = 0; c < nt; ++c) {
-      if (!mbar_wait(&s.sfull[t], c & 1, abort)) {
+      if (!warp_wait(&s.sfull[t], c & 1)) {
         ok = false;
         break;
       }
-      __syncwarp();
       tc_fence_after();
       float x0[64], x1[64];
       tmem_ld64(ts, x0);
@@ -264,8 +280,7 @@ __global__ void __launch_bounds__(kWAttnThreads, 1)
       if (lane == 0) mbar_arrive(&s.pready[t]);
     }
     if (ok && nt > 0) {
-      ok = mbar_wait(&s.ofull[t], 0, abort);
-      __syncwarp();
+      ok = warp_wait(&s.ofull[t], 0);
       tc_fence_after();
       const bool live = ok && row < tile_rows(t);
       __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.out) +

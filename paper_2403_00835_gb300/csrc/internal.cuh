@@ -120,6 +120,7 @@ struct AttnArgs {
   void* out;          // [T][H*hd] (+ lo plane in the bf16 engine)
   size_t plane_out;
   int T;
+  int hold;  // test hook: 1 + the key chunk at which the wide kernel's issuer gives up (0: none)
   int* err;
 };
 

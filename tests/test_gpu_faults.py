@@ -95,6 +95,35 @@ def test_hold_barrier_rejects_bad_phase(tiny):
         eng.close()
 
 
+@pytest.mark.parametrize("chunk", [0, 2])
+def test_wide_attention_timeout_unwinds(tiny, chunk):
+    """The wide attention's softmax warps run out of time together (one lane
+    waits for its warp), before any chunk and between two; the context then
+    computes what it computed before."""
+    cfg, w = tiny
+    lib = _hooks()
+    lib.cllm_test_hold_attention.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.cllm_test_hold_attention.restype = ctypes.c_int
+    assert lib.cllm_test_hold_attention(None, 0) == -1
+    prompts = syn.make_prompts(cfg.vocab, [500], seed=85)
+    guesses = syn.make_guesses(cfg.vocab, 1, 8, seed=86)
+    eng = engine_for(cfg, w, max_batch=1, max_seq=520, max_block=8)
+    try:
+        head = eng.prefill(prompts)
+        ref = eng.jacobi_step(guesses, want_logits=True)
+        assert lib.cllm_test_hold_attention(eng._h, -2) == -1
+        assert lib.cllm_test_hold_attention(eng._h, chunk) == 0
+        with pytest.raises(CllmError) as e:
+            eng.prefill(prompts)
+        assert e.value.status == CLLM_ETIMEOUT
+        assert lib.cllm_test_hold_attention(eng._h, -1) == 0
+        np.testing.assert_array_equal(eng.prefill(prompts), head)
+        r = eng.jacobi_step(guesses, want_logits=True)
+        np.testing.assert_array_equal(r["logits"], ref["logits"])
+    finally:
+        eng.close()
+
+
 @pytest.mark.parametrize("rows", [64, 16])
 def test_split_timeout_leaves_no_counts_behind(tiny, rows):
     """The down projection's tiles (K = 688) are cut over three ranges.  One
