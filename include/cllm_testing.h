@@ -95,6 +95,16 @@ int cllm_test_hold_barrier(cllm_ctx *ctx, int phase);
 int cllm_test_hold_attention(cllm_ctx *ctx, int chunk);
 
 /*
+ * The same for the per-phase weight GEMMs on CTA pairs: the loading thread of
+ * each pair's even CTA stops before its chunk `chunk` (of those beyond the
+ * ring's stages: a CTA with fewer is not affected), as if its wait had run out,
+ * while the odd CTA's goes on for up to a ring.  The call returns
+ * CLLM_ETIMEOUT.  -1 disarms.  Drops the captured graphs.  EINVAL on a null
+ * ctx or chunk < -1.
+ */
+int cllm_test_hold_gemm(cllm_ctx *ctx, int chunk);
+
+/*
  * The same for the split-K waits of launches of up to 256 rows: every weight
  * tile's arrival count is set to `count`.  With -1 the first contributor of a
  * tile that is cut over several ranges waits for one arrival more than there

@@ -237,6 +237,7 @@ struct cllm_ctx {
   int trace_phase = -1;  // profiling: phase whose MMA stage arrivals are traced
   int hold_phase = -1;   // test hook: grid barrier that cannot open (bounded-wait path)
   int hold_attn = 0;     // test hook: 1 + the chunk at which the wide attention stops
+  int hold_gemm = 0;     // test hook: 1 + the chunk at which a pair's even producer stops
   bool step_logits = false;  // the step graph being built stores the LM head's logits
   std::map<std::tuple<int, int, int, int, int, unsigned long long, int, int, int, int>, GraphEntry>
       graphs;
@@ -340,6 +341,7 @@ GemmArgs tc_gemm_args(cllm_ctx* c, int mtiles, int M, int K, int T, EpiArgs& e, 
   g.lo_rows = c->Tcap;
   g.l2_ahead = kL2AheadDefault;
   g.pre_stages = 1 << 20;
+  g.hold = c->hold_gemm;
   const Part p = plan_group(mtiles, K, T, c->sms);
   g.gshift = kGroupShift;
   g.mtiles = p.mtiles;
@@ -371,6 +373,7 @@ cudaError_t gemm(cllm_ctx* c, cudaStream_t s, bool pdl, int kind, int mtiles, in
   g.lo_rows = c->Tcap;
   g.l2_ahead = kL2AheadDefault;
   g.pre_stages = 1 << 20;
+  g.hold = c->hold_gemm;
   cudaError_t err;
   if (!c->bf16) {
     g.mtiles = mtiles;
@@ -2189,6 +2192,12 @@ extern "C" int cllm_test_hold_barrier(cllm_ctx* c, int phase) {
 extern "C" int cllm_test_hold_attention(cllm_ctx* c, int chunk) {
   if (!c || chunk < -1) return CLLM_EINVAL;
   c->hold_attn = chunk + 1;
+  return drop_graphs(c);
+}
+
+extern "C" int cllm_test_hold_gemm(cllm_ctx* c, int chunk) {
+  if (!c || chunk < -1) return CLLM_EINVAL;
+  c->hold_gemm = chunk + 1;
   return drop_graphs(c);
 }
 

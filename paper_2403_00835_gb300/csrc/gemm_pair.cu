@@ -73,6 +73,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
   P.abort = abort_flag;
   P.jflag = abort_flag + 1;
+  int* issued = abort_flag + 2;  // chunks this CTA's producer has loaded
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t r = cluster_ctarank();
   const bool leader = r == 0;
@@ -110,11 +111,11 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   // have no odd tile (its loads are zero fill, its epilogue stores nothing)
   int c0, c1;
   cta_range(g, cta & ~1, c0, c1);
+  const uint32_t b_rows = static_cast<uint32_t>(Cfg::STACKED ? g.bn : g.bn / 2);
+  const uint32_t cta_bytes = Cfg::A_BYTES + (Cfg::STACKED ? 1u : 2u) * b_rows * kBK * 2;  // a chunk, one CTA
 
   if (warp == 0) {
     if (lane == 0) {
-      const uint32_t b_rows = static_cast<uint32_t>(Cfg::STACKED ? g.bn : g.bn / 2);
-      const uint32_t stage_bytes = 2u * (Cfg::A_BYTES + (Cfg::STACKED ? 1u : 2u) * b_rows * kBK * 2);
       int u = c0 / g.kchunks, ka = c0 - u * g.kchunks, kb = ka, mt = tile_of(g, u, cta);
       auto load_a = [&](int st) {
         uint8_t* dst = ring + st * Cfg::STAGE_BYTES;
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       // weights of the first stages do not depend on the previous kernel
       const int n = c1 - c0, pre = min(n, S);
       for (int j = 0; j < pre; ++j) {
-        if (leader) mbar_arrive_expect_tx(&P.full[j], stage_bytes);
+        if (leader) mbar_arrive_expect_tx(&P.full[j], 2 * cta_bytes);
         load_a(j);
       }
       pdl_wait();
@@ -160,8 +161,9 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       int j = pre;
       uint32_t ph = 0;
       for (int st = 0; j < n; ++j) {
+        if (leader && g.hold == j + 1) break;  // test hook: as if the wait had run out
         if (!mbar_wait(&P.empty[st], ph, P.abort)) break;
-        if (leader) mbar_arrive_expect_tx(&P.full[st], stage_bytes);
+        if (leader) mbar_arrive_expect_tx(&P.full[st], 2 * cta_bytes);
         load_a(st);
         load_b(st);
         if (++st == S) {
@@ -170,6 +172,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
       }
       // every load of the pair has landed (bounded) before the CTAs may leave
+      *issued = j;
       if (leader)
         for (int i = max(0, j - S); i < j; ++i) mbar_wait(&P.full[i % S], (i / S) & 1, nullptr);
     }
@@ -232,6 +235,9 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   cluster_arrive();
   cluster_wait();
   tc_fence_after();
+  if (threadIdx.x == 0 && leader && *issued < c1 - c0)
+    pair_land_peer(P.full, S, *issued, mapa_smem(issued, 1), cta_bytes);
+  __syncwarp();
   if (warp == 1) tmem_dealloc_pair(P.tmem, 512);
   cluster_arrive();
   cluster_wait();

@@ -76,6 +76,7 @@ struct WideSmem {
   uint64_t full[kWStages], empty[kWStages], tfull, tempty, drain;
   uint32_t tmem;
   int abort_flag;
+  int issued;  // chunks this CTA's producer has loaded
   int ok[2];  // [0] the accumulator wait's result, [1] this cluster finishes the unit
 };
 
@@ -375,6 +376,8 @@ __global__ void __launch_bounds__(kWThreads, 1)
   pdl_launch_dependents();
 
   WideWork work(g, cluster, gridDim.x / 2);
+  const int n_chunks = work.chunks();
+  const uint32_t cta_bytes = 2 * kWATile + static_cast<uint32_t>(g.bn) * kBK * 2;  // a chunk, one CTA
   Segment sg;
   int first, last;
   // first token and this CTA's first row of unit u (512 rows; GATEUP: 256 features)
@@ -387,7 +390,6 @@ __global__ void __launch_bounds__(kWThreads, 1)
   if (warp < 4) {
     setmaxnreg_dec<kWRegsLow>();
     if (warp == 0 && lane == 0) {
-      const uint32_t stage_bytes = 2u * (2 * kWATile + static_cast<uint32_t>(g.bn) * kBK * 2);
       // Position of the next chunk to be loaded; a unit's coordinates are
       // worked out once (this one thread's divisions for every chunk took
       // longer than the chunk's MMAs: QKV at 2048 rows 323 instead of 257 us).
@@ -433,12 +435,12 @@ __global__ void __launch_bounds__(kWThreads, 1)
         tma_load_2d_pair(ring + st * kWStage + 2 * kWATile, &mB, &s.full[st], p.k * kBK, p.tok);
       };
       // weights of the first stages do not depend on the previous kernel
-      const int n = work.chunks(), pre = min(n, kWStages);
+      const int n = n_chunks, pre = min(n, kWStages);
       Pos pa{work, {}, 0, 0, 0};
       seek(pa);
       Pos pb = pa;
       for (int j = 0; j < pre; ++j, advance(pa)) {
-        if (leader) mbar_arrive_expect_tx(&s.full[j], stage_bytes);
+        if (leader) mbar_arrive_expect_tx(&s.full[j], 2 * cta_bytes);
         load_a(pa, j);
       }
       pdl_wait();
@@ -446,8 +448,9 @@ __global__ void __launch_bounds__(kWThreads, 1)
       int j = pre;
       uint32_t ph = 0;  // parity of the use before this one
       for (int st = 0; j < n; ++j) {
+        if (leader && g.hold == j + 1) break;  // test hook: as if the wait had run out
         if (!mbar_wait(&s.empty[st], ph, abort)) break;
-        if (leader) mbar_arrive_expect_tx(&s.full[st], stage_bytes);
+        if (leader) mbar_arrive_expect_tx(&s.full[st], 2 * cta_bytes);
         load_a(pa, st);
         load_b(pa, st);
         advance(pa);
@@ -457,6 +460,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
         }
       }
       // every load of the pair has landed (bounded) before the CTAs may leave
+      s.issued = j;
       if (leader)
         for (int i = max(0, j - kWStages); i < j; ++i)
           mbar_wait(&s.full[i % kWStages], (i / kWStages) & 1, nullptr);
@@ -599,6 +603,9 @@ __global__ void __launch_bounds__(kWThreads, 1)
   cluster_arrive();
   cluster_wait();
   tc_fence_after();
+  if (threadIdx.x == 0 && leader && s.issued < n_chunks)
+    pair_land_peer(s.full, kWStages, s.issued, mapa_smem(&s.issued, 1), cta_bytes);
+  __syncwarp();
   if (warp == 1) tmem_dealloc_pair(tmem, 512);
   cluster_arrive();
   cluster_wait();

@@ -91,6 +91,7 @@ struct GemmArgs {
   int rows_q, rows_qk;  // QKV: first rows of the K and V sections (weight-map select)
   int lo_rows;          // row offset of the activations' lo plane in the B map
   int l2_ahead;         // weight tiles per CTA prefetched into L2 before the PDL wait
+  int hold;             // test hook: 1 + the chunk at which a pair's even producer gives up (0: none)
   int pre_stages;       // weight tiles issued before the phase's dependency is met (<= ring)
   float* partial;       // [units*maxc][bn][128] split-K partial tiles
   int* tickets;         // [units] arrival counters (self-resetting)

@@ -366,6 +366,11 @@ __device__ __forceinline__ uint32_t mapa_smem(const void* p, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
   return a;
 }
+__device__ __forceinline__ int ld_cluster_int(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
 // Arrive on a barrier of another CTA of the cluster (address from mapa_smem).
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
@@ -414,6 +419,19 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
       " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar) & 0xFEFFFFFFu)
       : "memory");
+}
+
+// Loads of a pair's odd CTA that its even CTA never posted: a producer that gave
+// up at chunk `mine` may have left its peer up to a ring ahead.  The even CTA
+// (after a cluster barrier, the peer still there) posts their bytes, stage by
+// stage, and waits (bounded) until they have landed.
+__device__ __forceinline__ void pair_land_peer(uint64_t* full, int stages, int mine, uint32_t peer_issued,
+                                               uint32_t peer_bytes) {
+  const int theirs = ld_cluster_int(peer_issued);
+  for (int i = mine; i < theirs; ++i) {
+    mbar_arrive_expect_tx(&full[i % stages], peer_bytes);
+    mbar_wait(&full[i % stages], (i / stages) & 1, nullptr);
+  }
 }
 
 // hi + lo of two accumulators: 16 fp32 columns at each of four tensor-memory

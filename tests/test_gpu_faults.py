@@ -124,6 +124,42 @@ def test_wide_attention_timeout_unwinds(tiny, chunk):
         eng.close()
 
 
+@pytest.mark.parametrize("n", [100, 200, 300])
+def test_pair_gemm_timeout_unwinds(n):
+    """One CTA of each pair stops loading while the other goes on: the pair
+    leaves only when both CTAs' copies have landed, and the context then
+    computes what it computed before.  A vocabulary of 40000 gives the LM head
+    more chunks per CTA than the ring has stages (both widths of the pair
+    kernel, and the one of more than 256 rows)."""
+    from dataclasses import replace
+    cfg = replace(syn.TINY_BF16, vocab=40000)
+    w = syn.weights_to(syn.make_weights(cfg, seed=7, device="cpu"), "cuda")
+    lib = _hooks()
+    lib.cllm_test_hold_gemm.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.cllm_test_hold_gemm.restype = ctypes.c_int
+    assert lib.cllm_test_hold_gemm(None, 6) == -1
+    prompts = syn.make_prompts(cfg.vocab, [20], seed=87)
+    guesses = syn.make_guesses(cfg.vocab, 1, n, seed=88)
+    eng = engine_for(cfg, w, max_batch=1, max_seq=2 * n + 30, max_block=n)
+    try:
+        head = eng.prefill(prompts)
+        ref = eng.jacobi_step(guesses, want_logits=True)
+        assert not eng.uses_persistent(n)
+        assert lib.cllm_test_hold_gemm(eng._h, -2) == -1
+        for chunk in (6, 7):
+            eng.prefill(prompts)
+            assert lib.cllm_test_hold_gemm(eng._h, chunk) == 0
+            with pytest.raises(CllmError) as e:
+                eng.jacobi_step(guesses)
+            assert e.value.status == CLLM_ETIMEOUT, chunk
+            assert lib.cllm_test_hold_gemm(eng._h, -1) == 0
+            np.testing.assert_array_equal(eng.prefill(prompts), head)
+            r = eng.jacobi_step(guesses, want_logits=True)
+            np.testing.assert_array_equal(r["logits"], ref["logits"])
+    finally:
+        eng.close()
+
+
 @pytest.mark.parametrize("rows", [64, 16])
 def test_split_timeout_leaves_no_counts_behind(tiny, rows):
     """The down projection's tiles (K = 688) are cut over three ranges.  One
