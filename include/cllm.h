@@ -266,7 +266,8 @@ int cllm_decode_read_stats(cllm_ctx *ctx, cllm_accept_stats *out, int64_t *acc_h
  * one kernel per phase.  Until the option is set the library takes the
  * persistent kernel where it is the faster of the two: for blocks of fewer than
  * 64 rows with at most about one attention item (16 rows of a head against 512
- * keys) per SM at the sequences' committed lengths.  Both paths compute
+ * keys) per SM at the sequences' committed lengths when the call begins
+ * (cllm_decode_run chooses once per call).  Both paths compute
  * bit-identical results.  Takes effect for graphs captured after the call.
  * Returns CLLM_OK or EINVAL (unknown option).
  */

@@ -200,11 +200,12 @@ struct cllm_ctx {
   AttnMaps attn_maps{};     // bf16 engine: tensor maps of the attention tiles
   bool attn_maps_ok = false;
   int traj_cap = 0;
-  int* status_host = nullptr;  // pinned: slots of 4 ints {active, committed, device error, -}
+  // pinned: 2 slots of 4 ints {active, committed, device error, -}, then [max_batch] committed lengths
+  int* status_host = nullptr;
   cudaEvent_t iter_ev[2] = {nullptr, nullptr};
   // host state
   int B = 0;
-  std::vector<int> lens, Lh;
+  std::vector<int> lens, Lh;  // prompt lengths; committed lengths as of the last call
   bool prefilled = false;
   bool dec_active = false;
   int dec_n = 0, dec_max_new = 0;
@@ -1417,7 +1418,7 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
       rc = CLLM_ENOMEM;
       break;
     }
-    if (alloc_injected_failure() || cudaMallocHost(&c->status_host, 32) != cudaSuccess) {
+    if (alloc_injected_failure() || cudaMallocHost(&c->status_host, 32 + 4 * a.max_batch) != cudaSuccess) {
       rc = CLLM_ENOMEM;
       break;
     }
@@ -1767,9 +1768,14 @@ extern "C" int cllm_decode_run(cllm_ctx* c, int max_iters, int* iters_run, int64
       ++queued;
     }
   }
-  // a queued iteration past the end committed nothing; let it finish
-  e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "stream sync");
+  // a queued iteration past the end committed nothing; let it finish.  The
+  // committed lengths come back with it: the path rule and the capacity check
+  // of the next call go by them.
+  int* lens_host = c->status_host + 8;
+  e = cudaMemcpyAsync(lens_host, c->Ld, static_cast<size_t>(c->B) * sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "committed lengths");
+  c->Lh.assign(lens_host, lens_host + c->B);
   if (iters_run) *iters_run = it;
   if (committed) *committed = com;
   return CLLM_OK;

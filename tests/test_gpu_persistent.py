@@ -2,6 +2,8 @@
 barriers between phases) against the one-kernel-per-phase path: same work
 split, reductions and epilogues, so predictions, gaps, accepted counts,
 committed lengths and decoded tokens must be bit-identical."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 
@@ -126,3 +128,39 @@ def test_persistent_dataflow_flags_bit_identical(tiny_bf16, n):
     np.testing.assert_array_equal(a["logits"], b["logits"])
     np.testing.assert_array_equal(a["next"], b["next"])
     np.testing.assert_array_equal(a["accepted"], b["accepted"])
+
+
+def test_path_rule_follows_the_committed_lengths():
+    """The library's own choice goes by the lengths a decode has reached, not by
+    the prompt's: 32 heads at 16 rows have 160 attention items up to 2560 keys
+    (at most 171 run persistent on 152 SMs) and 192 beyond.  A decode that
+    crosses the line gives the same tokens as one that stays on either path."""
+    cfg = replace(syn.TINY_BF16, n_heads=32, n_kv_heads=4)
+    w = syn.make_weights(cfg, seed=21, device="cuda")
+    n, max_new = 16, 24
+    prompts = syn.make_prompts(cfg.vocab, [2540], seed=22)
+    guesses = syn.make_guesses(cfg.vocab, 1, n, seed=23)
+    runs = []
+    for choice in (None, True, False):
+        eng = engine_for(cfg, w, max_batch=1, max_seq=2540 + max_new + 2 * n, max_block=n)
+        try:
+            if choice is not None:
+                eng.set_persistent(choice)
+            eng.prefill(prompts)
+            eng.decode_begin(n, max_new, seed=24)
+            if choice is None:
+                assert eng.uses_persistent(n)
+            done, _ = eng.decode_run(1)
+            while done < max_new and eng.committed_lengths()[0] <= 2560 - n:
+                done += eng.decode_run(1)[0]
+            if choice is None:
+                assert not eng.uses_persistent(n)
+            eng.decode_run(max_new + 1)
+            tokens, iters = eng.decode_read()
+            step = eng.jacobi_step(guesses, want_logits=True)
+            runs.append((tokens, iters, step["logits"]))
+        finally:
+            eng.close()
+    for other in runs[1:]:
+        for a, b in zip(runs[0], other):
+            np.testing.assert_array_equal(a, b)
