@@ -263,7 +263,7 @@ int cllm_decode_read_stats(cllm_ctx *ctx, cllm_accept_stats *out, int64_t *acc_h
  * persistent kernel (one CTA per SM; phases embed, per layer QKV / attention /
  * O / gate-up / down, LM head, accept, separated by grid barriers).  Supported
  * when B*n <= 128 and head_dim is 64 or 128.  1 = wherever it is supported, 0 =
- * one kernel per phase.  Until the option is set the library takes the
+ * one kernel per phase, -1 (default) = the library's choice: the
  * persistent kernel where it is the faster of the two: for blocks of fewer than
  * 64 rows with at most about one attention item (16 rows of a head against 512
  * keys) per SM at the sequences' committed lengths when the call begins

@@ -309,6 +309,10 @@ class Engine:
     def set_persistent(self, on: bool):
         _check(self._lib.cllm_set_option(self._h, CLLM_OPT_PERSISTENT, 1 if on else 0), "cllm_set_option")
 
+    def set_persistent_auto(self):
+        """Back to the default: the library chooses the path."""
+        _check(self._lib.cllm_set_option(self._h, CLLM_OPT_PERSISTENT, -1), "cllm_set_option")
+
     def set_l2_pairs(self, pairs: int):
         _check(self._lib.cllm_set_option(self._h, CLLM_OPT_L2_PAIRS, int(pairs)), "cllm_set_option")
 

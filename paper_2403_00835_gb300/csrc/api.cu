@@ -1870,7 +1870,7 @@ extern "C" int cllm_ar_decode(cllm_ctx* c, int B, const int32_t* tokens, const i
 extern "C" int cllm_set_option(cllm_ctx* c, int option, int value) {
   if (!c) return CLLM_EINVAL;
   if (option == CLLM_OPT_PERSISTENT) {
-    c->persistent = value != 0 ? 1 : 0;
+    c->persistent = value < 0 ? -1 : (value != 0 ? 1 : 0);
     return CLLM_OK;
   }
   if (option == CLLM_OPT_L2_PAIRS) {

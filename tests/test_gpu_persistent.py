@@ -164,3 +164,19 @@ def test_path_rule_follows_the_committed_lengths():
     for other in runs[1:]:
         for a, b in zip(runs[0], other):
             np.testing.assert_array_equal(a, b)
+
+
+def test_path_choice_can_be_given_back_to_the_library(tiny_bf16):
+    cfg, eng = tiny_bf16
+    eng.set_persistent_auto()
+    eng.prefill(syn.make_prompts(cfg.vocab, [32, 17, 45, 20], seed=13))
+    try:
+        default = {n: eng.uses_persistent(n) for n in (1, 15, 16)}
+        assert default[15] and not default[16]  # 60 and 64 rows
+        for on in (True, False):
+            eng.set_persistent(on)
+            assert all(eng.uses_persistent(n) == on for n in default)
+            eng.set_persistent_auto()
+            assert {n: eng.uses_persistent(n) for n in default} == default
+    finally:
+        eng.set_persistent_auto()
