@@ -145,6 +145,10 @@ int cllm_test_plan_gemm(int mtiles, int K, int T, int sms, int *out);
  */
 int cllm_test_plan_group(int mtiles, int K, int T, int sms, int *out);
 
+/* The SM count that cllm_test_plan_group's split uses in this context: at most
+ * two for each CTA pair that can be resident at once.  EINVAL on a null ctx. */
+int cllm_test_split_sms(cllm_ctx *ctx);
+
 /*
  * Host-only: the work split of a launch of more than 256 tokens over `clusters`
  * CTA pairs (any T >= 1 is planned).  out[6] = {row units (512 weight rows;

@@ -171,6 +171,7 @@ struct cllm_ctx {
   float* gemm_part = nullptr;
   size_t gemm_part_elems = 0;
   int* tickets = nullptr;
+  int split_sms = 0;           // SMs that launches of up to 256 rows are split over
   int wide_clusters = 0;       // wide GEMM launches: resident clusters
   float* wide_part = nullptr;  // two split-K partials per CTA
   int* wide_tickets = nullptr;
@@ -343,7 +344,7 @@ GemmArgs tc_gemm_args(cllm_ctx* c, int mtiles, int M, int K, int T, EpiArgs& e, 
   g.l2_ahead = kL2AheadDefault;
   g.pre_stages = 1 << 20;
   g.hold = c->hold_gemm;
-  const Part p = plan_group(mtiles, K, T, c->sms);
+  const Part p = plan_group(mtiles, K, T, c->split_sms);
   g.gshift = kGroupShift;
   g.mtiles = p.mtiles;
   g.ntiles = p.ntiles;
@@ -1227,7 +1228,7 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
   if (!c) return CLLM_ENOMEM;
   c->arch = a;
   c->dev = dev;
-  c->sms = prop.multiProcessorCount;
+  c->sms = c->split_sms = prop.multiProcessorCount;
   c->bf16 = a.dtype == CLLM_BF16;
   c->esz = c->bf16 ? 2 : 4;
   c->planes = c->bf16 ? 2 : 1;
@@ -1301,6 +1302,14 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
           step_persistent_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess ||
           gemm_wide_set_attributes_acc() != cudaSuccess || gemm_pair_set_attributes() != cudaSuccess ||
           attention_wide_set_attributes() != cudaSuccess) {
+        rc = CLLM_ECUDA;
+        break;
+      }
+      // A tile's first contributor waits for the others, so every pair of a
+      // launch must be resident: an SM that no pair can use gets no share (the
+      // GB300's 152 SMs hold 76 pairs).  plan_group needs one group of 4 CTAs.
+      c->split_sms = std::min(c->sms, 2 * gemm_pair_clusters());
+      if (c->split_sms < 4) {
         rc = CLLM_ECUDA;
         break;
       }
@@ -1381,7 +1390,7 @@ extern "C" int cllm_create(const cllm_arch* arch, const cllm_weights* w, void* c
     size_t need = 0;
     c->max_mtiles = 0;
     for (int i = 0; i < 5; ++i) {
-      const Part p = plan_group(mt_list[i], k_list[i], std::min(256, bn_split), c->sms);
+      const Part p = plan_group(mt_list[i], k_list[i], std::min(256, bn_split), c->split_sms);
       need = std::max(need, static_cast<size_t>(mt_list[i]) * p.maxc * p.bn * kBM);
       c->max_mtiles = std::max(c->max_mtiles, mt_list[i]);
     }
@@ -2234,6 +2243,8 @@ extern "C" int cllm_test_plan_group(int mtiles, int K, int T, int sms, int* out)
   std::memcpy(out, v, sizeof v);
   return CLLM_OK;
 }
+
+extern "C" int cllm_test_split_sms(cllm_ctx* c) { return c ? c->split_sms : CLLM_EINVAL; }
 
 extern "C" int cllm_test_plan_wide(int gate_up, int M, int K, int T, int clusters, int split, int* out) {
   if (!out || M < 1 || K < 1 || T < 1 || clusters < 1) return CLLM_EINVAL;

@@ -13,6 +13,8 @@
 // (gemm_roles.cuh): every output element is the same sums in the same order,
 // so a token's bits do not depend on which kernel the launch's width selects.
 #define CLLM_EPI_GROUPS 1
+#include <algorithm>
+
 #include "act.cuh"
 #include "epilogue.cuh"
 #include "gemm_roles.cuh"
@@ -261,6 +263,25 @@ cudaError_t gemm_pair_set_attributes() {
   if ((err = pair_set_kind<EPI_RESID>()) != cudaSuccess) return err;
   return pair_set_kind<EPI_ARGMAX>();
 }
+
+template <int BN>
+static int pair_clusters() {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3(2 * 64);
+  cfg.blockDim = dim3(kPairThreads);
+  cfg.dynamicSmemBytes = pair_smem_bytes<BN>();
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<EPI_QKV, BN>, &cfg) == cudaSuccess ? n : 0;
+}
+
+int gemm_pair_clusters() { return std::min(pair_clusters<128>(), pair_clusters<256>()); }
 
 template <int KIND, int BN>
 static cudaError_t launch_pair_one(const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int grid, cudaStream_t s,

@@ -307,6 +307,7 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, 
 cudaError_t launch_gemm_pair(int kind, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int grid,
                              cudaStream_t s, bool pdl);
 cudaError_t gemm_pair_set_attributes();
+int gemm_pair_clusters();  // pairs that can be resident at once (0: an error); after the attributes are set
 inline int pair_box_rows(int bn) { return bn <= 128 ? bn : bn / 2; }
 
 // Wide launches (T > 256, gemm_wide.cu): units of 512 weight rows (gate/up:

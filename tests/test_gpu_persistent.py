@@ -2,6 +2,7 @@
 barriers between phases) against the one-kernel-per-phase path: same work
 split, reductions and epilogues, so predictions, gaps, accepted counts,
 committed lengths and decoded tokens must be bit-identical."""
+import ctypes
 from dataclasses import replace
 
 import numpy as np
@@ -10,6 +11,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from paper_2403_00835_gb300 import synthetic as syn
+from paper_2403_00835_gb300.cllm import load
 from tests.parity_util import engine_for
 
 pytestmark = pytest.mark.gpu
@@ -180,3 +182,15 @@ def test_path_choice_can_be_given_back_to_the_library(tiny_bf16):
             assert {n: eng.uses_persistent(n) for n in default} == default
     finally:
         eng.set_persistent_auto()
+
+
+def test_pair_launches_are_split_over_resident_pairs(tiny_bf16):
+    """Shared tiles' first contributors wait for the others: the split must not
+    be made for more CTAs than can be resident as pairs."""
+    _, eng = tiny_bf16
+    f = load().cllm_test_split_sms
+    f.argtypes, f.restype = [ctypes.c_void_p], ctypes.c_int
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = f(eng._h)
+    assert 4 <= n <= sms and n % 2 == 0
+    assert f(None) == -1

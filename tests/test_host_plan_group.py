@@ -68,6 +68,12 @@ def test_group_split_keeps_the_7b_shares(mtiles, K, share):
     assert plan(mtiles, K, 16)["cpc"] == share
 
 
+@pytest.mark.parametrize("sms", [152, 151, 150, 148, 7, 4])
+def test_group_split_launches_no_more_ctas_than_it_is_given(sms):
+    for mtiles, K in SHAPES:
+        assert plan(mtiles, K, 16, sms)["grid"] <= sms
+
+
 def test_bad_arguments_are_rejected():
     f = load().cllm_test_plan_group
     f.argtypes = [ctypes.c_int] * 4 + [ctypes.POINTER(ctypes.c_int)]
