@@ -13,9 +13,9 @@ extern "C" {
 #endif
 
 /*
- * The bf16 weight-streaming GEMM of the block forward (tcgen05/TMA kernel with
- * its work split and fixed-order split-K reduction) with the residual
- * epilogue:  Y[t][m] += sum_k W[m][k] * (Xhi[t][k] + Xlo[t][k])  for t < T, m < M.
+ * The bf16 weight GEMM of the block forward for T tokens (the tcgen05/TMA kernel
+ * that the engine launches, on CTA pairs, with its work split and fixed-order
+ * split-K reduction) with the residual epilogue:  Y[t][m] += sum_k W[m][k] * (Xhi[t][k] + Xlo[t][k])  for t < T, m < M.
  * W: device bf16 [M][K]; X: device bf16 [2][x_rows][K], the hi plane then the
  * lo plane of the activations (the engine carries every GEMM input as
  * hi = bf16(v), lo = bf16(v - hi)), x_rows >= T rounded up to 16 (and >= 256
@@ -31,9 +31,8 @@ int cllm_test_gemm_bf16(const void *W, const void *X, float *Y, int M, int K, in
  * Timing of the same kernel in a chain: `iters` launches captured in one CUDA
  * graph, launch i reading weights W + (i % n_w) * w_stride_bytes (distinct
  * matrices keep the chain from being served by L2), all accumulating into Y.
- * pdl: launch with programmatic dependent launch; l2_ahead: weight tiles per
- * CTA prefetched into L2 before waiting on the previous launch (the engine
- * uses 16).  T <= 256.  The graph runs once to warm up, then once timed with
+ * pdl: launch with programmatic dependent launch; l2_ahead >= 0 has no effect
+ * (the kernel starts its weight stream before it waits).  T <= 256.  The graph runs once to warm up, then once timed with
  * CUDA events; *us_per_launch = elapsed / iters.  Returns a CLLM_* status.
  */
 int cllm_test_gemm_bf16_timed(const void *W, long long w_stride_bytes, int n_w, const void *X,

@@ -1955,103 +1955,116 @@ extern "C" int cllm_committed_lengths(cllm_ctx* c, int32_t* lens_out) {
 
 #include "../../include/cllm_testing.h"
 
-extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M, int K, int T,
-                                   int x_rows) {
-  if (!W || !X || !Y || M < 128 || M % 128 || K < 8 || K % 8 || T < 1) return CLLM_EINVAL;
-  if (x_rows < round_up(T, 16) || (T > 256 && x_rows < 256)) return CLLM_EINVAL;
-  if (!aligned16(W) || !aligned16(X) || !aligned16(Y)) return CLLM_EINVAL;
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
-    return CLLM_ECUDA;
-  if (prop.major != 10 || prop.minor != 3) return CLLM_EUNSUPPORTED;
-  if (!get_encode() || gemm_tc_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess ||
-      gemm_wide_set_attributes_acc() != cudaSuccess)
-    return CLLM_ECUDA;
-  const int mtiles = M / kBM;
-  const Part p = plan_gemm(mtiles, K, T, prop.multiProcessorCount);
-  const int ldt = round_up(T, 16);
-  const bool wide = T > 256;
+namespace {
+// One weight GEMM of the block forward on its own, with the residual epilogue:
+// the work split, maps and scratch of the launch that the engine would make
+// for T tokens.
+struct TestGemm {
+  bool wide = false;
+  Part p{};
   WidePlan w{};
-  if (wide) {
-    const int clusters = gemm_wide_clusters();
-    if (clusters < 1) return CLLM_ECUDA;
-    w = plan_wide(EPI_RESID, M, K, T, clusters, true);
-  }
-  GemmMaps maps{};
-  if (!make_map(&maps.a0, W, K, M, kBM) || !make_map(&maps.b, X, K, 2 * x_rows, wide ? w.bn : p.bn))
-    return CLLM_EINVAL;
-  maps.a1 = maps.a2 = maps.a0;
+  GemmArgs g{};
+  EpiArgs e{};
   std::vector<void*> tmp;
-  auto alloc = [&](size_t bytes) -> void* {
+  ~TestGemm() {
+    for (void* v : tmp) cudaFree(v);
+  }
+  void* alloc(size_t bytes) {
     void* v = nullptr;
-    if (cudaMalloc(&v, bytes) != cudaSuccess || cudaMemset(v, 0, bytes) != cudaSuccess) return nullptr;
+    if (cudaMalloc(&v, bytes) != cudaSuccess) return nullptr;
     tmp.push_back(v);
-    return v;
-  };
-  int rc = CLLM_OK;
-  do {
-    const size_t ctas = static_cast<size_t>(w.clusters) * 2;
-    float* part = static_cast<float*>(
-        alloc(wide ? 2 * ctas * kWidePartFloats * 4 : static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
-    int* tickets = static_cast<int*>(alloc(wide ? ctas * 4 : mtiles * 4));
-    int* err = static_cast<int*>(alloc(16));
-    float* ssq = static_cast<float*>(alloc(static_cast<size_t>(mtiles) * ldt * 4));
-    void* xg = alloc(static_cast<size_t>(T) * M * 2 * 2);
-    __nv_bfloat16* ones = static_cast<__nv_bfloat16*>(alloc(static_cast<size_t>(M) * 2));
-    if (!part || !tickets || !err || !ssq || !xg || !ones) {
-      rc = CLLM_ENOMEM;
-      break;
-    }
-    std::vector<__nv_bfloat16> h1(M, __float2bfloat16(1.f));
-    if (cudaMemcpy(ones, h1.data(), M * 2, cudaMemcpyHostToDevice) != cudaSuccess) {
-      rc = CLLM_ECUDA;
-      break;
-    }
-    GemmArgs g{};
+    return cudaMemset(v, 0, bytes) == cudaSuccess ? v : nullptr;
+  }
+  int init(float* Y, int M, int K, int T, int x_rows) {
+    int dev = 0;
+    cudaDeviceProp prop;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
+      return CLLM_ECUDA;
+    if (prop.major != 10 || prop.minor != 3) return CLLM_EUNSUPPORTED;
+    if (!get_encode() || gemm_pair_set_attributes() != cudaSuccess || gemm_wide_set_attributes() != cudaSuccess ||
+        gemm_wide_set_attributes_acc() != cudaSuccess)
+      return CLLM_ECUDA;
+    const int mtiles = M / kBM, ldt = round_up(T, 16);
+    wide = T > 256;
     g.M = M;
     g.K = K;
     g.T = T;
-    g.mtiles = p.mtiles;
-    g.ntiles = p.ntiles;
-    g.kchunks = p.kchunks;
-    g.cpc = p.cpc;
-    g.bn = p.bn;
-    g.maxc = p.maxc;
     g.rows_q = M;
     g.rows_qk = M;
     g.lo_rows = x_rows;
     g.l2_ahead = kL2AheadDefault;
     g.pre_stages = 1 << 20;
-    if (wide) w.apply(g);
-    g.partial = part;
-    g.tickets = tickets;
-    g.err = err;
-    EpiArgs e{};
+    size_t parts, tickets;  // floats, ints
+    if (wide) {
+      const int clusters = gemm_wide_clusters();
+      if (clusters < 1) return CLLM_ECUDA;
+      w = plan_wide(EPI_RESID, M, K, T, clusters, true);
+      w.apply(g);
+      tickets = static_cast<size_t>(w.clusters) * 2;
+      parts = 2 * tickets * kWidePartFloats;
+    } else {
+      const int sms = std::min(prop.multiProcessorCount, 2 * gemm_pair_clusters());
+      if (sms < 4) return CLLM_ECUDA;
+      p = plan_group(mtiles, K, T, sms);
+      g.gshift = kGroupShift;
+      g.mtiles = p.mtiles;
+      g.ntiles = p.ntiles;
+      g.kchunks = p.kchunks;
+      g.cpc = p.cpc;
+      g.bn = p.bn;
+      g.maxc = p.maxc;
+      tickets = mtiles;
+      parts = static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM;
+    }
+    g.partial = static_cast<float*>(alloc(parts * 4));
+    g.tickets = static_cast<int*>(alloc(tickets * 4));
+    g.err = static_cast<int*>(alloc(16));
     e.T = T;
     e.ldt = ldt;
     e.x = Y;
-    e.xg = xg;
+    e.xg = alloc(static_cast<size_t>(T) * M * 2 * 2);
+    __nv_bfloat16* ones = static_cast<__nv_bfloat16*>(alloc(static_cast<size_t>(M) * 2));
     e.gnext = ones;
     e.plane_x = static_cast<size_t>(T) * M;
-    e.ssq_out = ssq;
+    e.ssq_out = static_cast<float*>(alloc(static_cast<size_t>(mtiles) * ldt * 4));
     e.d = M;
-    e.err = err;
-    const cudaError_t le = wide ? launch_gemm_wide(EPI_RESID, maps, g, e, w.clusters, 0, false)
-                                : launch_gemm_tc(EPI_RESID, p.bn_max, maps, g, e, p.grid, 0, false);
-    if (le != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
-      rc = CLLM_ECUDA;
-      break;
-    }
+    e.err = g.err;
+    if (!g.partial || !g.tickets || !g.err || !e.xg || !ones || !e.ssq_out) return CLLM_ENOMEM;
+    const std::vector<__nv_bfloat16> h1(M, __float2bfloat16(1.f));
+    return cudaMemcpy(ones, h1.data(), M * 2, cudaMemcpyHostToDevice) == cudaSuccess ? CLLM_OK : CLLM_ECUDA;
+  }
+  bool maps(GemmMaps& m, const void* W, const void* X) const {
+    const uint64_t k = static_cast<uint64_t>(g.K);
+    if (!make_map(&m.a0, W, k, g.M, kBM) ||
+        !make_map(&m.b, X, k, 2 * static_cast<uint64_t>(g.lo_rows), wide ? w.bn : pair_box_rows(p.bn)))
+      return false;
+    m.a1 = m.a2 = m.a0;
+    return true;
+  }
+  cudaError_t launch(const GemmMaps& m, cudaStream_t s, bool pdl) const {
+    return wide ? launch_gemm_wide(EPI_RESID, m, g, e, w.clusters, s, pdl)
+                : launch_gemm_pair(EPI_RESID, m, g, e, p.grid, s, pdl);
+  }
+  int device_status() const {
     int herr = 0;
-    if (cudaMemcpy(&herr, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) {
-      rc = CLLM_ECUDA;
-      break;
-    }
-    if (herr) rc = (herr & DERR_TIMEOUT) ? CLLM_ETIMEOUT : CLLM_EDEVICE;
-  } while (0);
-  for (void* v : tmp) cudaFree(v);
-  return rc;
+    if (cudaMemcpy(&herr, g.err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return CLLM_ECUDA;
+    return herr == 0 ? CLLM_OK : (herr & DERR_TIMEOUT) ? CLLM_ETIMEOUT : CLLM_EDEVICE;
+  }
+};
+}  // namespace
+
+extern "C" int cllm_test_gemm_bf16(const void* W, const void* X, float* Y, int M, int K, int T,
+                                   int x_rows) {
+  if (!W || !X || !Y || M < 128 || M % 128 || K < 8 || K % 8 || T < 1) return CLLM_EINVAL;
+  if (x_rows < round_up(T, 16) || (T > 256 && x_rows < 256)) return CLLM_EINVAL;
+  if (!aligned16(W) || !aligned16(X) || !aligned16(Y)) return CLLM_EINVAL;
+  TestGemm t;
+  const int rc = t.init(Y, M, K, T, x_rows);
+  if (rc != CLLM_OK) return rc;
+  GemmMaps m{};
+  if (!t.maps(m, W, X)) return CLLM_EINVAL;
+  if (t.launch(m, 0, false) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return CLLM_ECUDA;
+  return t.device_status();
 }
 
 extern "C" int cllm_test_gemm_bf16_timed(const void* W, long long w_stride_bytes, int n_w,
@@ -2061,110 +2074,41 @@ extern "C" int cllm_test_gemm_bf16_timed(const void* W, long long w_stride_bytes
       T > 256 || iters < 1 || n_w < 1 || l2_ahead < 0)
     return CLLM_EINVAL;
   if (x_rows < round_up(T, 16)) return CLLM_EINVAL;
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess)
-    return CLLM_ECUDA;
-  if (prop.major != 10 || prop.minor != 3) return CLLM_EUNSUPPORTED;
-  if (!get_encode() || gemm_tc_set_attributes() != cudaSuccess) return CLLM_ECUDA;
-  const int mtiles = M / kBM;
-  const Part p = plan_gemm(mtiles, K, T, prop.multiProcessorCount);
-  const int ldt = round_up(T, 16);
+  TestGemm t;
+  int rc = t.init(Y, M, K, T, x_rows);
+  if (rc != CLLM_OK) return rc;
   std::vector<GemmMaps> maps(n_w);
-  for (int i = 0; i < n_w; ++i) {
-    const char* wi = static_cast<const char*>(W) + static_cast<long long>(i) * w_stride_bytes;
-    if (!make_map(&maps[i].a0, wi, K, M, kBM) || !make_map(&maps[i].b, X, K, 2 * x_rows, p.bn))
+  for (int i = 0; i < n_w; ++i)
+    if (!t.maps(maps[i], static_cast<const char*>(W) + static_cast<long long>(i) * w_stride_bytes, X))
       return CLLM_EINVAL;
-    maps[i].a1 = maps[i].a2 = maps[i].a0;
-  }
-  std::vector<void*> tmp;
-  auto alloc = [&](size_t bytes) -> void* {
-    void* v = nullptr;
-    if (cudaMalloc(&v, bytes) != cudaSuccess || cudaMemset(v, 0, bytes) != cudaSuccess) return nullptr;
-    tmp.push_back(v);
-    return v;
-  };
-  int rc = CLLM_OK;
   cudaStream_t s = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
+  rc = CLLM_ECUDA;
   do {
-    float* part = static_cast<float*>(alloc(static_cast<size_t>(mtiles) * p.maxc * p.bn * kBM * 4));
-    int* tickets = static_cast<int*>(alloc(mtiles * 4));
-    int* err = static_cast<int*>(alloc(16));
-    float* ssq = static_cast<float*>(alloc(static_cast<size_t>(mtiles) * ldt * 4));
-    void* xg = alloc(static_cast<size_t>(T) * M * 2 * 2);
-    void* ones = alloc(static_cast<size_t>(M) * 2);
-    if (!part || !tickets || !err || !ssq || !xg || !ones) {
-      rc = CLLM_ENOMEM;
-      break;
-    }
     if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
-      rc = CLLM_ECUDA;
+        cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess ||
+        cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
       break;
-    }
-    GemmArgs g{};
-    g.M = M;
-    g.K = K;
-    g.T = T;
-    g.mtiles = p.mtiles;
-    g.ntiles = p.ntiles;
-    g.kchunks = p.kchunks;
-    g.cpc = p.cpc;
-    g.bn = p.bn;
-    g.maxc = p.maxc;
-    g.rows_q = M;
-    g.rows_qk = M;
-    g.lo_rows = x_rows;
-    g.l2_ahead = l2_ahead;
-    g.pre_stages = 1 << 20;
-    g.partial = part;
-    g.tickets = tickets;
-    g.err = err;
-    EpiArgs e{};
-    e.T = T;
-    e.ldt = ldt;
-    e.x = Y;
-    e.xg = xg;
-    e.gnext = ones;
-    e.plane_x = static_cast<size_t>(T) * M;
-    e.ssq_out = ssq;
-    e.d = M;
-    e.err = err;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-      rc = CLLM_ECUDA;
-      break;
-    }
     cudaError_t le = cudaSuccess;
-    for (int i = 0; i < iters && le == cudaSuccess; ++i)
-      le = launch_gemm_tc(EPI_RESID, p.bn_max, maps[i % n_w], g, e, p.grid, s, pdl != 0);
-    cudaError_t ce = cudaStreamEndCapture(s, &graph);
-    if (le != cudaSuccess || ce != cudaSuccess ||
-        cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) {
-      rc = CLLM_ECUDA;
-      break;
-    }
+    for (int i = 0; i < iters && le == cudaSuccess; ++i) le = t.launch(maps[i % n_w], s, pdl != 0);
+    const cudaError_t ce = cudaStreamEndCapture(s, &graph);
+    if (le != cudaSuccess || ce != cudaSuccess || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) break;
     if (cudaGraphLaunch(exec, s) != cudaSuccess || cudaEventRecord(e0, s) != cudaSuccess ||
         cudaGraphLaunch(exec, s) != cudaSuccess || cudaEventRecord(e1, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-      rc = CLLM_ECUDA;
+        cudaStreamSynchronize(s) != cudaSuccess)
       break;
-    }
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
     *us_per_launch = ms * 1000.f / iters;
-    int herr = 0;
-    cudaMemcpy(&herr, err, 4, cudaMemcpyDeviceToHost);
-    if (herr) rc = (herr & DERR_TIMEOUT) ? CLLM_ETIMEOUT : CLLM_EDEVICE;
+    rc = t.device_status();
   } while (0);
   if (exec) cudaGraphExecDestroy(exec);
   if (graph) cudaGraphDestroy(graph);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (s) cudaStreamDestroy(s);
-  for (void* v : tmp) cudaFree(v);
   return rc;
 }
 
