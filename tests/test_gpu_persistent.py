@@ -194,3 +194,25 @@ def test_pair_launches_are_split_over_resident_pairs(tiny_bf16):
     n = f(eng._h)
     assert 4 <= n <= sms and n % 2 == 0
     assert f(None) == -1
+
+
+@pytest.mark.parametrize("B,n", [(1, 64), (4, 16), (1, 65), (2, 50), (1, 128), (8, 16)])
+def test_wider_blocks_have_the_same_logits_on_both_paths(B, n):
+    """64 to 128 rows, the widths at which the library's own choice is the pair
+    kernels: every logit bit for bit against the persistent kernel's."""
+    cfg = syn.TINY_BF16
+    w = syn.make_weights(cfg, seed=0, device="cuda")
+    prompts = syn.make_prompts(cfg.vocab, [11 + 9 * b for b in range(B)], seed=31)
+    guesses = syn.make_guesses(cfg.vocab, B, n, seed=32)
+    eng = engine_for(cfg, w, max_batch=B, max_seq=300, max_block=n)
+    try:
+        out = []
+        for on in (True, False):
+            eng.set_persistent(on)
+            eng.prefill(prompts)
+            assert eng.uses_persistent(n) == on
+            out.append(eng.jacobi_step(guesses, want_gap=True, want_logits=True))
+        for key in out[0]:
+            np.testing.assert_array_equal(out[0][key], out[1][key])
+    finally:
+        eng.close()

@@ -103,9 +103,9 @@ def test_wide_prefill_matches_oracle(hd, kv, ffn, lens):
         head, gap, _ = orc.prefill(s, p)
         if gap >= FLAG_GAP:
             assert heads[b] == head
-            st = orc.jacobi_step(s, [head] + list(guesses[b][1:]), len(p), keep_logits=True)
-            ok, worst = logits_ok(r["logits"][b], st.logits, "bf16")
-            assert ok, (b, worst)
+        st = orc.jacobi_step(s, [int(heads[b])] + list(guesses[b][1:]), len(p), keep_logits=True)
+        ok, worst = logits_ok(r["logits"][b], st.logits, "bf16")
+        assert ok, (b, worst)
         s.close()
 
 
