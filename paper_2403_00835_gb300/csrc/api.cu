@@ -341,8 +341,6 @@ GemmArgs tc_gemm_args(cllm_ctx* c, int mtiles, int M, int K, int T, EpiArgs& e, 
   g.tickets = c->tickets;
   g.partial = c->gemm_part;
   g.lo_rows = c->Tcap;
-  g.l2_ahead = kL2AheadDefault;
-  g.pre_stages = 1 << 20;
   g.hold = c->hold_gemm;
   const Part p = plan_group(mtiles, K, T, c->split_sms);
   g.gshift = kGroupShift;
@@ -373,8 +371,6 @@ cudaError_t gemm(cllm_ctx* c, cudaStream_t s, bool pdl, int kind, int mtiles, in
   g.tickets = c->tickets;
   g.partial = c->gemm_part;
   g.lo_rows = c->Tcap;
-  g.l2_ahead = kL2AheadDefault;
-  g.pre_stages = 1 << 20;
   g.hold = c->hold_gemm;
   cudaError_t err;
   if (!c->bf16) {
@@ -1992,8 +1988,6 @@ struct TestGemm {
     g.rows_q = M;
     g.rows_qk = M;
     g.lo_rows = x_rows;
-    g.l2_ahead = kL2AheadDefault;
-    g.pre_stages = 1 << 20;
     size_t parts, tickets;  // floats, ints
     if (wide) {
       const int clusters = gemm_wide_clusters();

@@ -24,8 +24,8 @@ namespace cllm {
 // ---------------------------------------------------------------------------------
 
 // Columns whose per-token epilogue inputs (RMSNorm scale, position, sequence)
-// are prepared once per launch / phase (launches with more tokens prepare them
-// per 16-column chunk).
+// are prepared once per launch / phase (the launches that run tc_epilogue have no
+// more; the fp32 GEMM prepares them per 16-column chunk).
 constexpr int kEpiPrepMax = 256;
 
 struct EpiSmem {
@@ -110,6 +110,9 @@ __device__ __forceinline__ void epi_ssq_quad(const EpiArgs& e, int t, int part, 
 template <int KIND>
 __device__ void epi_prepare(const EpiArgs& e, int r, EpiSmem& s, int gi = 0, int ng = 1) {
   s.prepared = 0;
+  // (guards the tables: no launch that comes here has more columns.  The branch
+  // stays also because the compiler schedules the pair kernels better with it:
+  // 64 rows 3.98 ms, without it 4.03.)
   if (e.T > kEpiPrepMax) {
     epi_sync();
     return;

@@ -1,6 +1,6 @@
-// The weight-streaming GEMM on its own (the allocation-free entry point and the
-// test hooks; the engine's launches run on CTA pairs, gemm_pair.cu and
-// gemm_wide.cu, or inside the persistent kernel).
+// The weight-streaming GEMM on its own (the allocation-free entry point up to 256
+// tokens; the engine's launches run on CTA pairs, gemm_pair.cu and gemm_wide.cu,
+// or inside the persistent kernel).  Y[t][m] += D[m][t]: the residual add alone.
 //
 //   D[m][t] = sum_k W[m][k] * X[t][k]      (W: [M][K] weights, X: [T][K] activations)
 //
@@ -42,7 +42,7 @@ constexpr int kSoloRedSlots = 2;  // split-K partial blocks staged per reduction
 // Epilogue groups: at 256 token columns one accumulator fills tensor memory,
 // so the MMAs of a CTA's next unit wait for the whole epilogue of the last
 // one (16 chunks); a second group of 4 warps halves that wait.
-template <int KIND, int BNMAX>
+template <int BNMAX>
 constexpr int solo_groups() { return BNMAX == 256 ? 2 : 1; }
 
 constexpr size_t kSoloGroupBytes = (sizeof(EpiSmem) + 15) / 16 * 16 + kSoloRedSlots * kRedSlotBytes;
@@ -50,8 +50,7 @@ constexpr size_t kSoloGroupBytes = (sizeof(EpiSmem) + 15) / 16 * 16 + kSoloRedSl
 template <int BNMAX>
 constexpr size_t solo_smem_bytes() {
   using Cfg = SoloCfg<BNMAX>;
-  constexpr int groups = BNMAX == 256 ? 2 : 1;  // room for two groups at 256 columns
-  return 1024 + static_cast<size_t>(Cfg::STAGES) * Cfg::STAGE_BYTES + groups * kSoloGroupBytes + 16 +
+  return 1024 + static_cast<size_t>(Cfg::STAGES) * Cfg::STAGE_BYTES + solo_groups<BNMAX>() * kSoloGroupBytes + 16 +
          tc_bar_bytes(Cfg::STAGES) + 16;
 }
 constexpr size_t kSmemLimit = 227 * 1024 - 256;  // minus static shared memory
@@ -59,25 +58,22 @@ static_assert(solo_smem_bytes<32>() <= kSmemLimit && solo_smem_bytes<64>() <= kS
                   solo_smem_bytes<128>() <= kSmemLimit && solo_smem_bytes<256>() <= kSmemLimit,
               "per-GEMM kernel shared memory over the 227 KB limit");
 
-template <int KIND, int BNMAX>
-__global__ void __launch_bounds__(64 + 128 * solo_groups<KIND, BNMAX>(), 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
-                   const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB,
-                   const GemmArgs g, const EpiArgs e) {
+template <int BNMAX>
+__global__ void __launch_bounds__(64 + 128 * solo_groups<BNMAX>(), 1)
+    gemm_tc_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, const GemmArgs g,
+                   const EpiArgs e) {
   using Cfg = SoloCfg<BNMAX>;
-  constexpr int NG = solo_groups<KIND, BNMAX>();
+  constexpr int NG = solo_groups<BNMAX>();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base =
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // [ring][per group: EpiSmem, staging slots][barriers][shared flags, 16 bytes]
   uint8_t* groups = base + Cfg::STAGES * Cfg::STAGE_BYTES;
-  uint8_t* bars = groups + (BNMAX == 256 ? 2 : 1) * kSoloGroupBytes;
+  uint8_t* bars = groups + NG * kSoloGroupBytes;
   int* jflag = reinterpret_cast<int*>(bars + tc_bar_bytes(Cfg::STAGES));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0 && lane == 0) {
-    tma_prefetch_desc(&mA0);
-    tma_prefetch_desc(&mA1);
-    tma_prefetch_desc(&mA2);
+    tma_prefetch_desc(&mA);
     tma_prefetch_desc(&mB);
   }
   TcPipe P = tc_pipe_init<Cfg, NG>(base, bars);
@@ -90,9 +86,7 @@ __global__ void __launch_bounds__(64 + 128 * solo_groups<KIND, BNMAX>(), 1)
   cta_range(g, blockIdx.x, c0, c1);
   if (warp == 0) {
     if (lane == 0) {
-      int idx = 0, issued = 0;
-      tc_produce<KIND, Cfg>(P, idx, issued, g, &mA0, &mA1, &mA2, &mB, c0, c1, blockIdx.x, PdlDep{});
-      tc_produce_drain<Cfg>(P, issued);
+      tc_produce_drain<Cfg>(P, tc_produce<Cfg>(P, g, &mA, &mB, c0, c1, blockIdx.x));
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -110,7 +104,7 @@ __global__ void __launch_bounds__(64 + 128 * solo_groups<KIND, BNMAX>(), 1)
     Pg.red = reinterpret_cast<float*>(mine + (sizeof(EpiSmem) + 15) / 16 * 16);
     int acc = 0;
     uint32_t accph = 0;
-    tc_epilogue<KIND, Cfg, NG>(Pg, acc, accph, g, e, c0, c1, blockIdx.x, es);
+    tc_epilogue<EPI_ACC, Cfg, NG>(Pg, acc, accph, g, e, c0, c1, blockIdx.x, es);
   }
   tc_pipe_release<Cfg>(P);
   if (threadIdx.x == 0 && *P.abort) atomicOr(g.err, DERR_TIMEOUT);
@@ -120,31 +114,23 @@ __global__ void __launch_bounds__(64 + 128 * solo_groups<KIND, BNMAX>(), 1)
 // launchers
 // ---------------------------------------------------------------------------------
 
-template <int KIND, int BN>
+template <int BN>
 static cudaError_t set_attr_one() {
-  cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<KIND, BN>,
+  cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(solo_smem_bytes<BN>()));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(gemm_tc_kernel<KIND, BN>,
+  return cudaFuncSetAttribute(gemm_tc_kernel<BN>,
                               cudaFuncAttributePreferredSharedMemoryCarveout,
                               static_cast<int>(cudaSharedmemCarveoutMaxShared));
 }
 
-cudaError_t gemm_tc_set_attributes() {
-  cudaError_t err;
-  if ((err = set_attr_one<EPI_RESID, 32>()) != cudaSuccess) return err;
-  if ((err = set_attr_one<EPI_RESID, 64>()) != cudaSuccess) return err;
-  if ((err = set_attr_one<EPI_RESID, 128>()) != cudaSuccess) return err;
-  return set_attr_one<EPI_RESID, 256>();
-}
-
-cudaError_t gemm_tc_set_attributes_acc(int bn_max) {
+cudaError_t gemm_tc_set_attributes(int bn_max) {
   switch (bn_max) {
-    case 32: return set_attr_one<EPI_ACC, 32>();
-    case 64: return set_attr_one<EPI_ACC, 64>();
-    case 128: return set_attr_one<EPI_ACC, 128>();
-    default: return set_attr_one<EPI_ACC, 256>();
+    case 32: return set_attr_one<32>();
+    case 64: return set_attr_one<64>();
+    case 128: return set_attr_one<128>();
+    default: return set_attr_one<256>();
   }
 }
 
@@ -161,32 +147,22 @@ static void fill_launch(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3
   cfg.numAttrs = 1;
 }
 
-template <int KIND, int BN>
+template <int BN>
 static cudaError_t launch_tc_one(const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int grid,
                                  cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  fill_launch(cfg, attr, dim3(grid), dim3(64 + 128 * solo_groups<KIND, BN>()), solo_smem_bytes<BN>(), s, pdl);
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<KIND, BN>, m.a0, m.a1, m.a2, m.b, g, e);
+  fill_launch(cfg, attr, dim3(grid), dim3(64 + 128 * solo_groups<BN>()), solo_smem_bytes<BN>(), s, pdl);
+  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN>, m.a0, m.b, g, e);
 }
 
-template <int KIND>
-static cudaError_t launch_tc_kind(int bn_max, const GemmMaps& m, const GemmArgs& g,
-                                  const EpiArgs& e, int grid, cudaStream_t s, bool pdl) {
+cudaError_t launch_gemm_tc(int bn_max, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int grid,
+                           cudaStream_t s, bool pdl) {
   switch (bn_max) {
-    case 32: return launch_tc_one<KIND, 32>(m, g, e, grid, s, pdl);
-    case 64: return launch_tc_one<KIND, 64>(m, g, e, grid, s, pdl);
-    case 128: return launch_tc_one<KIND, 128>(m, g, e, grid, s, pdl);
-    case 256: return launch_tc_one<KIND, 256>(m, g, e, grid, s, pdl);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_gemm_tc(int kind, int bn_max, const GemmMaps& maps, const GemmArgs& g,
-                           const EpiArgs& e, int grid, cudaStream_t s, bool pdl) {
-  switch (kind) {
-    case EPI_RESID: return launch_tc_kind<EPI_RESID>(bn_max, maps, g, e, grid, s, pdl);
-    case EPI_ACC: return launch_tc_kind<EPI_ACC>(bn_max, maps, g, e, grid, s, pdl);
+    case 32: return launch_tc_one<32>(m, g, e, grid, s, pdl);
+    case 64: return launch_tc_one<64>(m, g, e, grid, s, pdl);
+    case 128: return launch_tc_one<128>(m, g, e, grid, s, pdl);
+    case 256: return launch_tc_one<256>(m, g, e, grid, s, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

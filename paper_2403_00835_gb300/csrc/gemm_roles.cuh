@@ -1,13 +1,12 @@
-// The three warp roles of the weight-streaming GEMM, as device functions that
-// carry their pipeline state across calls.  The stand-alone GEMM kernel runs one
-// phase; the persistent per-iteration kernel (its own producer and MMA roles)
-// runs many phases' epilogues back to back, and the CTA-pair kernel one.
+// The warp roles of the weight-streaming GEMM.  The stand-alone GEMM kernel uses
+// all three; the persistent per-iteration kernel and the CTA-pair kernel have
+// producers and MMA issuers of their own and share the epilogue, which carries
+// its pipeline state across the persistent kernel's phases.
 //
 //   producer (one thread): TMA of weight tiles (A, evict-first) and the
 //     activation tile's hi/lo planes (B, evict-last) into the stage ring.
 //     Weight tiles do not depend on earlier work, so they are issued before
-//     the phase's dependency (previous kernel / grid barrier) is satisfied;
-//     activation tiles only after.
+//     the previous kernel has finished; activation tiles only after.
 //   MMA issuer (one thread): tcgen05.mma M=128 into a TMEM accumulator pair.
 //   epilogue (warps 2..5, 128 threads): tcgen05.ld, split-K partials reduced in
 //     a fixed order by the tile's first contributor, fused epilogue (epilogue.cuh).
@@ -117,19 +116,7 @@ __device__ void tc_pipe_release(const TcPipe& P) {
   }
 }
 
-// ---- dependency policies --------------------------------------------------------
-
-// Standalone kernels: the previous kernel in the stream (programmatic
-// dependent launch); not pollable.
-struct PdlDep {
-  static constexpr bool kPollable = false;
-  __device__ bool ready() const { return false; }
-  __device__ bool wait(volatile int*) const {
-    pdl_wait();
-    return true;
-  }
-  __device__ void after() const {}
-};
+// ---- the persistent kernel's dependency ------------------------------------------
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
   unsigned v;
@@ -140,7 +127,6 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
 // Persistent kernel: grid barrier counter >= target (every CTA finished the
 // phases this one depends on).  Waits are bounded.
 struct GridDep {
-  static constexpr bool kPollable = true;
   const unsigned* counter;
   unsigned target;
   __device__ bool ready() const { return ld_acquire_gpu(counter) >= target; }
@@ -198,124 +184,41 @@ __device__ __forceinline__ void cta_range(const GemmArgs& g, int cta, int& c0, i
 
 // ---- producer -------------------------------------------------------------------------
 
-// Issue this CTA's chunks [c0, c1) of one GEMM phase.  `idx` counts chunks
-// issued so far (ring position).  Returns false if a bounded wait gave up.
-template <int KIND, class Cfg, class Dep>
-__device__ bool tc_produce(const TcPipe& P, int& idx, int& issued_b, const GemmArgs& g,
-                           const CUtensorMap* mA0, const CUtensorMap* mA1, const CUtensorMap* mA2,
-                           const CUtensorMap* mB, int c0, int c1, int cta, const Dep& dep) {
+// Issue this CTA's chunks [c0, c1) of a launch of its own (stand-alone GEMM: one
+// weight matrix).  Returns the number of chunks issued: fewer than asked for if
+// a bounded wait gave up.
+template <class Cfg>
+__device__ int tc_produce(const TcPipe& P, const GemmArgs& g, const CUtensorMap* mA, const CUtensorMap* mB, int c0,
+                          int c1, int cta) {
   constexpr int S = Cfg::STAGES;
-  const int n = c1 - c0;
-  if (n <= 0) {
-    if (!Dep::kPollable) dep.wait(P.abort);
-    return true;
-  }
+  const int n = c1 - c0, pre = min(n, S);
   const uint64_t pol_w = l2_policy_evict_first();
   const uint64_t pol_x = l2_policy_evict_last();
   const uint32_t b_bytes = 2u * static_cast<uint32_t>(g.bn) * kBK * 2;
   auto load_a = [&](int j, int st) {
     const int c = c0 + j;
     const int u = c / g.kchunks, k = c - u * g.kchunks;
-    const int mt = tile_of(g, u, cta);
-    uint8_t* dst = P.sA + st * Cfg::A_BYTES;
-    if (KIND == EPI_GATEUP) {
-      tma_load_2d(dst, mA0, &P.full[st], k * kBK, mt * 64, pol_w);
-      tma_load_2d(dst + Cfg::A_BYTES / 2, mA1, &P.full[st], k * kBK, mt * 64, pol_w);
-    } else if (KIND == EPI_QKV) {
-      const int row = mt * kBM;
-      if (row < g.rows_q)
-        tma_load_2d(dst, mA0, &P.full[st], k * kBK, row, pol_w);
-      else if (row < g.rows_qk)
-        tma_load_2d(dst, mA1, &P.full[st], k * kBK, row - g.rows_q, pol_w);
-      else
-        tma_load_2d(dst, mA2, &P.full[st], k * kBK, row - g.rows_qk, pol_w);
-    } else {
-      tma_load_2d(dst, mA0, &P.full[st], k * kBK, mt * kBM, pol_w);
-    }
+    mbar_arrive_expect_tx(&P.full[st], Cfg::A_BYTES + b_bytes);
+    tma_load_2d(P.sA + st * Cfg::A_BYTES, mA, &P.full[st], k * kBK, tile_of(g, u, cta) * kBM, pol_w);
   };
   auto load_b = [&](int j, int st) {
-    const int c = c0 + j;
-    const int k = c % g.kchunks;
+    const int k = (c0 + j) % g.kchunks;
     uint8_t* dst = P.sB + st * Cfg::B_BYTES;
     tma_load_2d(dst, mB, &P.full[st], k * kBK, 0, pol_x);
     tma_load_2d(dst + (Cfg::STACKED ? g.bn * kBK * 2 : Cfg::B_HALF), mB, &P.full[st], k * kBK, g.lo_rows,
                 pol_x);
   };
-  auto prefetch_l2 = [&](int j) {
-    const int c = c0 + j;
-    const int u = c / g.kchunks, k = c - u * g.kchunks;
-    const int mt = tile_of(g, u, cta);
-    if (KIND == EPI_GATEUP) {
-      tma_prefetch_l2_2d(mA0, k * kBK, mt * 64);
-      tma_prefetch_l2_2d(mA1, k * kBK, mt * 64);
-    } else if (KIND == EPI_QKV) {
-      const int row = mt * kBM;
-      if (row < g.rows_q)
-        tma_prefetch_l2_2d(mA0, k * kBK, row);
-      else if (row < g.rows_qk)
-        tma_prefetch_l2_2d(mA1, k * kBK, row - g.rows_q);
-      else
-        tma_prefetch_l2_2d(mA2, k * kBK, row - g.rows_qk);
-    } else {
-      tma_prefetch_l2_2d(mA0, k * kBK, mt * kBM);
-    }
-  };
-  // Weight tiles into free stages while the dependency is not satisfied; once
-  // the ring is full, the next l2_ahead tiles into L2 (once), so that HBM
-  // keeps streaming while the previous phase drains.
-  int j = 0;
-  bool open = Dep::kPollable ? dep.ready() : false;
-  bool prefetched = false;
-  uint64_t t0 = 0;
-  while (j < n && !open) {
-    const int gi = idx + j, st = gi % S;
-    if (j < g.pre_stages && mbar_try_wait(&P.empty[st], ((gi / S) & 1) ^ 1)) {
-      mbar_arrive_expect_tx(&P.full[st], Cfg::A_BYTES + b_bytes);
-      load_a(j, st);
-      ++j;
-      if (Dep::kPollable) open = dep.ready();
-      continue;
-    }
-    if (!Dep::kPollable) break;
-    if (!prefetched) {
-      for (int jj = j; jj < min(n, j + g.l2_ahead); ++jj) prefetch_l2(jj);
-      prefetched = true;
-    }
-    open = dep.ready();
-    if (open) break;
-    if (*P.abort) break;  // gave up: dep.wait below returns false at once
-    if (t0 == 0) {
-      t0 = globaltimer_ns();
-    } else if (globaltimer_ns() - t0 > kWaitBudgetNs) {
-      *P.abort = 1;
-      break;
-    }
-    __nanosleep(32);
-  }
-  const bool dep_ok = open || dep.wait(P.abort);
-  if (dep_ok) dep.after();
-  // Activation tiles of the stages issued so far.  (On a failed wait they are
-  // still issued -- in-bounds reads of stale data -- so that every stage this
-  // thread started completes and can be drained before the CTA exits.)
-  for (int jj = 0; jj < j; ++jj) load_b(jj, (idx + jj) % S);
-  issued_b = idx + j;
-  if (!dep_ok) {
-    idx += j;
-    return false;
-  }
-  for (; j < n; ++j) {
-    const int gi = idx + j, st = gi % S;
-    if (!mbar_wait(&P.empty[st], ((gi / S) & 1) ^ 1, P.abort)) {
-      idx += j;
-      return false;
-    }
-    mbar_arrive_expect_tx(&P.full[st], Cfg::A_BYTES + b_bytes);
+  // weights of the first stages do not depend on the previous kernel
+  for (int j = 0; j < pre; ++j) load_a(j, j);
+  pdl_wait();
+  for (int j = 0; j < pre; ++j) load_b(j, j);
+  for (int j = pre; j < n; ++j) {
+    const int st = j % S;
+    if (!mbar_wait(&P.empty[st], ((j / S) & 1) ^ 1, P.abort)) return j;
     load_a(j, st);
     load_b(j, st);
-    issued_b = gi + 1;
   }
-  idx += n;
-  return true;
+  return max(n, 0);
 }
 
 // Before exit: every fully issued stage has landed (bounded).
@@ -328,14 +231,8 @@ __device__ void tc_produce_drain(const TcPipe& P, int issued) {
 // ---- MMA issuer ------------------------------------------------------------------------
 
 template <class Cfg>
-__device__ bool tc_mma(const TcPipe& P, int& idx, int& acc, uint32_t& accph, const GemmArgs& g,
-                       int c0, int c1, unsigned long long* prof = nullptr, long long prof_stride = 0,
-                       unsigned long long* trace = nullptr) {
+__device__ bool tc_mma(const TcPipe& P, int& idx, int& acc, uint32_t& accph, const GemmArgs& g, int c0, int c1) {
   constexpr int S = Cfg::STAGES;
-  // optional profile: first and last stage arrival, largest gap between
-  // arrivals, and (trace) every arrival
-  unsigned long long t_first = 0, t_last = 0, gap = 0;
-  int ntrace = 0;
   const uint32_t idesc = idesc_bf16_f32(kBM, Cfg::STACKED ? 2 * g.bn : g.bn);
   int c = c0;
   Segment sg;
@@ -347,13 +244,6 @@ __device__ bool tc_mma(const TcPipe& P, int& idx, int& acc, uint32_t& accph, con
       const int st = idx % S;
       if (!mbar_wait(&P.full[st], (idx / S) & 1, P.abort)) return false;
       tc_fence_after();
-      if (prof != nullptr) {
-        const unsigned long long now = globaltimer_ns();
-        if (trace != nullptr && ntrace < kTraceCap) trace[ntrace++] = now;
-        if (t_first == 0) t_first = now;
-        else if (now - t_last > gap) gap = now - t_last;
-        t_last = now;
-      }
       const uint32_t a_addr = smem_u32(P.sA + st * Cfg::A_BYTES);
       const uint32_t b_addr = smem_u32(P.sB + st * Cfg::B_BYTES);
 #pragma unroll
@@ -372,11 +262,6 @@ __device__ bool tc_mma(const TcPipe& P, int& idx, int& acc, uint32_t& accph, con
       acc = 0;
       accph ^= 1;
     }
-  }
-  if (prof != nullptr) {
-    prof[0] = t_first;
-    prof[prof_stride] = t_last;
-    prof[2 * prof_stride] = gap;
   }
   return true;
 }

@@ -24,10 +24,6 @@ constexpr int kQTile = 16;       // query rows per attention tile
 constexpr int kBK = 64;          // K elements per pipeline stage (128 B of bf16)
 constexpr int kBM = 128;         // weight rows per tile (MMA M)
 constexpr int kEpiCols = 16;     // columns per epilogue chunk
-// Weight tiles per CTA prefetched into L2 ahead of the shared-memory ring by
-// the per-GEMM kernels.  Measured on chains of GEMM launches: it adds traffic
-// without shortening the chain, so it is off.
-constexpr int kL2AheadDefault = 0;
 
 // EPI_ACC (stand-alone GEMMs): x += D, without the next norm's input and statistics
 enum EpiKind : int { EPI_QKV = 0, EPI_GATEUP = 1, EPI_RESID = 2, EPI_ARGMAX = 3, EPI_ACC = 4 };
@@ -90,9 +86,7 @@ struct GemmArgs {
   int gshift;           // log2 of the tiles per group
   int rows_q, rows_qk;  // QKV: first rows of the K and V sections (weight-map select)
   int lo_rows;          // row offset of the activations' lo plane in the B map
-  int l2_ahead;         // weight tiles per CTA prefetched into L2 before the PDL wait
   int hold;             // test hook: 1 + the chunk at which a pair's even producer gives up (0: none)
-  int pre_stages;       // weight tiles issued before the phase's dependency is met (<= ring)
   float* partial;       // [units*maxc][bn][128] split-K partial tiles
   int* tickets;         // [units] arrival counters (self-resetting)
   // fp32 path only
@@ -336,8 +330,8 @@ cudaError_t launch_gemm_wide(int kind, const GemmMaps& m, const GemmArgs& g, con
                              cudaStream_t s, bool pdl);
 
 cudaError_t launch_embed(const EmbedArgs& a, int act_bf16, cudaStream_t s, bool pdl);
-cudaError_t launch_gemm_tc(int kind, int bn_max, const GemmMaps& maps, const GemmArgs& g,
-                           const EpiArgs& e, int grid, cudaStream_t s, bool pdl);
+cudaError_t launch_gemm_tc(int bn_max, const GemmMaps& m, const GemmArgs& g, const EpiArgs& e, int grid,
+                           cudaStream_t s, bool pdl);
 cudaError_t launch_attention(const AttnArgs& a, int grid, cudaStream_t s, bool pdl);
 // bf16 engine with tensor maps: Q, K and V tiles by TMA (kv_row0: the layer's
 // first cache row in the maps)
@@ -360,8 +354,7 @@ cudaError_t launch_gather_rows(const void* xg_src, const float* ssq_src, void* x
                                float* ssq_dst, const int* rows, int B, int d, int ldt_src,
                                int ldt_dst, size_t plane_src, size_t plane_dst, int act_bf16,
                                cudaStream_t s);
-cudaError_t gemm_tc_set_attributes();
-cudaError_t gemm_tc_set_attributes_acc(int bn_max);  // EPI_ACC, one column count
+cudaError_t gemm_tc_set_attributes(int bn_max);  // of one column count
 cudaError_t attention_set_attributes();
 size_t attention_smem_bytes(int hd);
 

@@ -86,7 +86,7 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
     const int clusters = gemm_wide_clusters();
     if (clusters < 1) return CLLM_ECUDA;
     w = plan_wide(EPI_ACC, M, K, T, clusters, false);
-  } else if (gemm_tc_set_attributes_acc(p.bn_max) != cudaSuccess) {
+  } else if (gemm_tc_set_attributes(p.bn_max) != cudaSuccess) {
     return CLLM_ECUDA;
   }
   GemmMaps maps{};
@@ -110,8 +110,6 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   g.rows_q = M;
   g.rows_qk = M;
   g.lo_rows = x_rows;
-  g.l2_ahead = kL2AheadDefault;  // as the allocating GEMM entry points
-  g.pre_stages = 1 << 20;
   if (wide) w.apply(g);
   g.partial = reinterpret_cast<float*>(sb);
   g.tickets = reinterpret_cast<int*>(sb + off_tick);
@@ -122,7 +120,7 @@ extern "C" int cllm_gemm_bf16_noalloc(const void* W, const void* X, float* Y, in
   e.d = M;
   e.err = g.err;
   const cudaError_t le = wide ? launch_gemm_wide(EPI_ACC, maps, g, e, w.clusters, s, false)
-                              : launch_gemm_tc(EPI_ACC, p.bn_max, maps, g, e, p.grid, s, false);
+                              : launch_gemm_tc(p.bn_max, maps, g, e, p.grid, s, false);
   if (le != cudaSuccess) return CLLM_ECUDA;
   int herr = 0;
   if (cudaMemcpyAsync(&herr, g.err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
