@@ -21,6 +21,16 @@
  *     thread-safe; calls on one context must not overlap.
  *   - Every call on a context synchronises its stream before returning
  *     (unless stated otherwise), so host outputs are valid on return.
+ *   - Several contexts may share a GPU, but their calls should not overlap in
+ *     time: launches of up to 256 rows (a block's B*n rows, the last rows of a
+ *     prefill) have CTAs that wait for one another, and two contexts' launches
+ *     that hold each other's SMs let those waits run out (2 s, CLLM_ETIMEOUT).
+ *     Launches of more rows, and the fp32 engine's, have no such waits.
+ *   - A call's results are a function of its inputs, bit for bit.  In the fp32
+ *     engine, and in the bf16 engine's launches of up to 256 rows, a row's
+ *     results do not depend on the rows that share its launch; above 256 rows
+ *     sums are cut to suit the launch's row count, so the same row may differ
+ *     in its last bits between launches of different width.
  */
 #ifndef CLLM_H
 #define CLLM_H

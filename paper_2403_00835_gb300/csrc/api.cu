@@ -912,14 +912,19 @@ int build_persistent(cllm_ctx* c, int mode, int B, int n, const int2* qtiles, in
 
 // Whether an iteration of B x n rows runs as the persistent kernel: where it is
 // supported and, unless the caller has chosen, faster than one kernel per
-// phase on CTA pairs.  (Both give the same bits.)  7B shape, 8 layers, us per iteration, persistent against pairs:
+// phase on CTA pairs.  (Both give the same bits.)  The sequences' lengths are
+// those of the last call's end, so a decode that has run past the line changes
+// path at its next call.  7B shape, 8 layers, us per iteration, persistent
+// against pairs:
 // the pairs fetch less activation data per weight tile, which decides from 64
 // rows on (64 rows 1081 / 1061, 96 1440 / 1169, 128 1692 / 1269; 48 rows 983 /
 // 1031); below that the persistent kernel saves the launches, until its one
 // CTA per SM has more than about a wave of attention items of up to 512 keys
 // (16 rows at 2048 keys, 160 items: 926 / 969; at 4096, 288: 1053 / 1017; 32
 // rows at 512 keys, 128: 951 / 973; at 1024, 192: 1033 / 981; 8 sequences at
-// 1024 keys, 768: 1300 / 1131).
+// 1024 keys, 768: 1300 / 1131).  A small decoder (2 layers, d_model 256) is
+// faster on the pairs on both sides of the line: 64 rows 154 / 115, 128 rows
+// 244 / 148, and 48 rows 134 / 109.
 bool persistent_ok(cllm_ctx* c, int B, int n) {
   // (the attention's K/V tensor maps address cache rows with 32-bit coordinates)
   if (!(c->bf16 && c->persistent != 0 && B * n <= 128 && 7 * c->NL + 7 <= kMaxStepMaps &&

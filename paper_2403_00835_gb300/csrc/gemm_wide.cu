@@ -34,14 +34,11 @@
 // other until the waits ran out.)
 //
 // Per launch at 2048 rows, 7B shape, against the single-CTA kernel: gate/up
-// 757 -> 384 us (1.93 PFLOP/s counting both planes: the power limit), QKV 555
-// -> 241, O and down together 511 -> 357; at 1024 rows gate/up 571 -> 302 (a
-// mean over 1024- and 2048-row launches).  Those were taken with two pairs of
-// a cluster sharing each weight tile by multicast loads; a pair now loads its
-// own, because the ranks of a replica run load this library too and a
-// multicast load has no place in a multi-GPU program.  4096-row prefill
-// (2 layers) 5.23 -> 5.53 ms, 500 rows 1.23 -> 1.25, 16 x 64 rows unchanged
-// (the pairs use all 152 SMs, clusters of 4 used 144).
+// 757 -> 405 us (1.82 PFLOP/s counting both planes: near the power limit), QKV
+// 555 -> 246, O and down together 511 -> 359.  Two pairs of a cluster sharing
+// each weight tile by multicast loads would take gate/up to 384 us (4096-row
+// prefill, 2 layers, 5.20 against 5.30 ms), but the ranks of a replica run load
+// this library too, and a multicast load has no place in a multi-GPU program.
 #include <float.h>
 #include <limits.h>
 
@@ -397,6 +394,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
         WideWork w;
         Segment sg;
         int k, row0, tok;
+        const CUtensorMap* m;  // QKV: the matrix that holds all of the CTA's rows (null: several do)
       };
       auto seek = [&](Pos& p) {
         int f, l;
@@ -404,6 +402,20 @@ __global__ void __launch_bounds__(kWThreads, 1)
         p.k = p.sg.k0;
         p.row0 = unit_row(p.sg.unit);
         p.tok = unit_tok(p.sg.unit) + (r ? g.lo_rows : 0);
+        if constexpr (KIND == EPI_QKV) {
+          // (row0 becomes the row within that matrix)
+          const int end = p.row0 + 2 * kBM;
+          p.m = nullptr;
+          if (end <= g.rows_q) {
+            p.m = &mA0;
+          } else if (p.row0 >= g.rows_qk) {
+            p.m = &mA2;
+            p.row0 -= g.rows_qk;
+          } else if (p.row0 >= g.rows_q && end <= g.rows_qk) {
+            p.m = &mA1;
+            p.row0 -= g.rows_q;
+          }
+        }
       };
       auto advance = [&](Pos& p) {
         if (++p.k == p.sg.k1) seek(p);
@@ -420,6 +432,19 @@ __global__ void __launch_bounds__(kWThreads, 1)
             tma_load_2d_pair(dst, m, bar, x, p.row0);
             tma_load_2d_pair(dst + kWATile / 2, m, bar, x, p.row0 + 64);
           } else if constexpr (KIND == EPI_QKV) {
+            // boxes of half a head: picking the matrix for every box took the
+            // one thread longer than the chunk's MMAs (2048 rows 334 us)
+            if (p.m != nullptr && half == 64) {
+              tma_load_2d_pair(dst, p.m, bar, x, p.row0 + a * 64);
+              tma_load_2d_pair(dst + 64 * kBK * 2, p.m, bar, x, p.row0 + 128 + a * 64);
+              continue;
+            }
+            if (p.m != nullptr) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                tma_load_2d_pair(dst + j * 32 * kBK * 2, p.m, bar, x, p.row0 + j * 64 + a * 32);
+              continue;
+            }
             for (int i = 0, y = p.row0 + a * half; i < kBM; i += half, y += e.hd) {
               uint8_t* d = dst + i * kBK * 2;
               if (y < g.rows_q) tma_load_2d_pair(d, &mA0, bar, x, y);
@@ -436,7 +461,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
       };
       // weights of the first stages do not depend on the previous kernel
       const int n = n_chunks, pre = min(n, kWStages);
-      Pos pa{work, {}, 0, 0, 0};
+      Pos pa{work, {}, 0, 0, 0, nullptr};
       seek(pa);
       Pos pb = pa;
       for (int j = 0; j < pre; ++j, advance(pa)) {
