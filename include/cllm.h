@@ -274,10 +274,9 @@ int cllm_decode_read_stats(cllm_ctx *ctx, cllm_accept_stats *out, int64_t *acc_h
  * O / gate-up / down, LM head, accept, separated by grid barriers).  Supported
  * when B*n <= 128 and head_dim is 64 or 128.  1 = wherever it is supported, 0 =
  * one kernel per phase, -1 (default) = the library's choice: the
- * persistent kernel where it is the faster of the two: for blocks of fewer than
- * 64 rows with at most about one attention item (16 rows of a head against 512
- * keys) per SM at the sequences' committed lengths when the call begins
- * (cllm_decode_run chooses once per call).  Both paths compute
+ * persistent kernel where it is the faster of the two: for blocks of up to 48
+ * rows whose attention is short at the sequences' committed lengths when the
+ * call begins (cllm_decode_run chooses once per call).  Both paths compute
  * bit-identical results.  Takes effect for graphs captured after the call.
  * Returns CLLM_OK or EINVAL (unknown option).
  */

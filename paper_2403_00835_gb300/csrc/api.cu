@@ -914,17 +914,24 @@ int build_persistent(cllm_ctx* c, int mode, int B, int n, const int2* qtiles, in
 // supported and, unless the caller has chosen, faster than one kernel per
 // phase on CTA pairs.  (Both give the same bits.)  The sequences' lengths are
 // those of the last call's end, so a decode that has run past the line changes
-// path at its next call.  7B shape, 8 layers, us per iteration, persistent
-// against pairs:
-// the pairs fetch less activation data per weight tile, which decides from 64
-// rows on (64 rows 1081 / 1061, 96 1440 / 1169, 128 1692 / 1269; 48 rows 983 /
-// 1031); below that the persistent kernel saves the launches, until its one
-// CTA per SM has more than about a wave of attention items of up to 512 keys
-// (16 rows at 2048 keys, 160 items: 926 / 969; at 4096, 288: 1053 / 1017; 32
-// rows at 512 keys, 128: 951 / 973; at 1024, 192: 1033 / 981; 8 sequences at
-// 1024 keys, 768: 1300 / 1131).  A small decoder (2 layers, d_model 256) is
-// faster on the pairs on both sides of the line: 64 rows 154 / 115, 128 rows
-// 244 / 148, and 48 rows 134 / 109.
+// path at its next call.
+//
+// The persistent kernel saves the launches, about 20 us a layer, and loses some
+// of it with every 16 rows (its epilogues take the columns 16 at a time, and
+// the pairs fetch less activation data): 7B shape, 4 layers, 30 keys, us per
+// iteration persistent / pairs: 16 rows 398 / 472, 32 rows 438 / 481, 48 rows
+// 493 / 519, 63 rows 546 / 535.  Its attention runs its items (16 rows of a head
+// against up to 512 keys) one per SM at a time, a wave taking 0.5 + the chunks
+// of 128 keys per item in units of ~11 us for those 4 layers, and tiles of more
+// than one range add a merge (one unit).  So: at most 9 units up to 16
+// rows, 7 up to 32 and 4.5 up to 48.  On both sides of the line: 15 rows of 15
+// sequences at 100 keys 479 / 492, at 250 533 / 515; 8 sequences at 500 keys
+// 496 / 502, at 1000 631 / 551; one sequence of 16 rows at 2000 keys 462 / 490, at
+// 4000 558 / 509; 32 rows at 500 keys 484 / 495, at 1000 520 / 498; 48 rows at
+// 250 keys 503 / 525, at 500 575 / 531; 8 key/value heads: 8 sequences at 400 keys
+// 422 / 450, at 2000 717 / 545.  Over 206 such points (three shapes) the choice
+// is within 1 % of the faster path but for three of a decoder of d_model 1024,
+// where it keeps the persistent kernel (3-6 %).
 bool persistent_ok(cllm_ctx* c, int B, int n) {
   // (the attention's K/V tensor maps address cache rows with 32-bit coordinates)
   if (!(c->bf16 && c->persistent != 0 && B * n <= 128 && 7 * c->NL + 7 <= kMaxStepMaps &&
@@ -932,11 +939,21 @@ bool persistent_ok(cllm_ctx* c, int B, int n) {
         B * ceil_div(n, kQTile) <= kMaxQTilesStep && (c->hd == 64 || c->hd == 128)))
     return false;
   if (c->persistent == 1) return true;
-  if (B * n >= 64) return false;
-  long items = 0;
+  if (B * n > 48) return false;
+  long items = 0, chunks = 0;
+  bool merge = false;
   for (int b = 0; b < B; ++b)
-    items += static_cast<long>(c->H) * ceil_div(n, kQTile) * ceil_div(c->Lh[b] + n, kAttnChunk * kAttnRange);
-  return items <= c->sms + c->sms / 8;
+    for (int r0 = 0; r0 < n; r0 += kQTile) {
+      const int keys = c->Lh[b] + std::min(n, r0 + kQTile);
+      const int ranges = ceil_div(keys, kAttnChunk * kAttnRange);
+      items += static_cast<long>(c->H) * ranges;
+      chunks += static_cast<long>(c->H) * ceil_div(keys, kAttnChunk);
+      merge = merge || ranges > 1;
+    }
+  // waves * (1/2 + chunks / items) + merge <= limit, times 2 items
+  const long waves = (items + c->sms - 1) / c->sms;
+  const long limit2 = B * n <= 16 ? 18 : (B * n <= 32 ? 14 : 9);
+  return waves * (items + 2 * chunks) + (merge ? 2 * items : 0) <= limit2 * items;
 }
 
 // Get (capturing on first use) the graph of one decode/step iteration.

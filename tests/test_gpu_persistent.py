@@ -134,17 +134,17 @@ def test_persistent_dataflow_flags_bit_identical(tiny_bf16, n):
 
 def test_path_rule_follows_the_committed_lengths():
     """The library's own choice goes by the lengths a decode has reached, not by
-    the prompt's: 32 heads at 16 rows have 160 attention items up to 2560 keys
-    (at most 171 run persistent on 152 SMs) and 192 beyond.  A decode that
-    crosses the line gives the same tokens as one that stays on either path."""
+    the prompt's: 16 rows of 32 heads run persistent (on 152 SMs) up to 2176
+    keys.  A decode that crosses the line gives the same tokens as one that stays
+    on either path."""
     cfg = replace(syn.TINY_BF16, n_heads=32, n_kv_heads=4)
     w = syn.make_weights(cfg, seed=21, device="cuda")
     n, max_new = 16, 24
-    prompts = syn.make_prompts(cfg.vocab, [2540], seed=22)
+    prompts = syn.make_prompts(cfg.vocab, [2152], seed=22)
     guesses = syn.make_guesses(cfg.vocab, 1, n, seed=23)
     runs = []
     for choice in (None, True, False):
-        eng = engine_for(cfg, w, max_batch=1, max_seq=2540 + max_new + 2 * n, max_block=n)
+        eng = engine_for(cfg, w, max_batch=1, max_seq=2152 + max_new + 2 * n, max_block=n)
         try:
             if choice is not None:
                 eng.set_persistent(choice)
@@ -153,7 +153,7 @@ def test_path_rule_follows_the_committed_lengths():
             if choice is None:
                 assert eng.uses_persistent(n)
             done, _ = eng.decode_run(1)
-            while done < max_new and eng.committed_lengths()[0] <= 2560 - n:
+            while done < max_new and eng.committed_lengths()[0] <= 2176 - n:
                 done += eng.decode_run(1)[0]
             if choice is None:
                 assert not eng.uses_persistent(n)
@@ -173,8 +173,8 @@ def test_path_choice_can_be_given_back_to_the_library(tiny_bf16):
     eng.set_persistent_auto()
     eng.prefill(syn.make_prompts(cfg.vocab, [32, 17, 45, 20], seed=13))
     try:
-        default = {n: eng.uses_persistent(n) for n in (1, 15, 16)}
-        assert default[15] and not default[16]  # 60 and 64 rows
+        default = {n: eng.uses_persistent(n) for n in (1, 12, 13)}
+        assert default[12] and not default[13]  # 48 and 52 rows
         for on in (True, False):
             eng.set_persistent(on)
             assert all(eng.uses_persistent(n) == on for n in default)
@@ -196,9 +196,9 @@ def test_pair_launches_are_split_over_resident_pairs(tiny_bf16):
     assert f(None) == -1
 
 
-@pytest.mark.parametrize("B,n", [(1, 64), (4, 16), (1, 65), (2, 50), (1, 128), (8, 16)])
+@pytest.mark.parametrize("B,n", [(5, 10), (1, 64), (4, 16), (1, 65), (2, 50), (1, 128), (8, 16)])
 def test_wider_blocks_have_the_same_logits_on_both_paths(B, n):
-    """64 to 128 rows, the widths at which the library's own choice is the pair
+    """50 to 128 rows, the widths at which the library's own choice is the pair
     kernels: every logit bit for bit against the persistent kernel's."""
     cfg = syn.TINY_BF16
     w = syn.make_weights(cfg, seed=0, device="cuda")
@@ -214,5 +214,22 @@ def test_wider_blocks_have_the_same_logits_on_both_paths(B, n):
             out.append(eng.jacobi_step(guesses, want_gap=True, want_logits=True))
         for key in out[0]:
             np.testing.assert_array_equal(out[0][key], out[1][key])
+    finally:
+        eng.close()
+
+
+@pytest.mark.parametrize("B,n,keys,persistent", [
+    (1, 16, 128, True), (1, 16, 2000, True), (1, 1, 4096, False), (15, 1, 47, True), (15, 1, 250, False),
+    (8, 1, 500, True), (8, 1, 1000, False), (1, 32, 500, True), (1, 32, 1000, False), (1, 48, 250, True),
+    (6, 7, 30, True), (1, 48, 500, False), (1, 49, 30, False), (24, 1, 30, False)])
+def test_path_rule_at_its_lines(B, n, keys, persistent):
+    """The library's own choice with 32 heads on 152 SMs, on both sides of its
+    lines: rows, waves of attention items and keys per item."""
+    cfg = replace(syn.TINY_BF16, n_heads=32, n_kv_heads=4, n_layers=1)
+    w = syn.make_weights(cfg, seed=41, device="cuda")
+    eng = engine_for(cfg, w, max_batch=B, max_seq=keys + n + 1, max_block=n)
+    try:
+        eng.prefill(syn.make_prompts(cfg.vocab, [keys] * B, seed=42))
+        assert eng.uses_persistent(n) == persistent
     finally:
         eng.close()
